@@ -85,7 +85,6 @@ struct CollideParams {
     double force[3] = {0.0, 0.0, 0.0}; // uniform body force (not from the paper), used by the forced kernels
     float beta_f = 0.0f;  // beta rounded to FP32 once on the host (no FP64 conversion per thread)
     float dunit_f = 0.0f; // R = W rho0 rounded to FP32: the unit of the deviation references c_i = k_i R
-    int pop_stream = 0;   // host side: the D3Q27 step loads with the evict-first policy (ld_pop)
 };
 
 // beta in the compute type.
@@ -155,11 +154,11 @@ __device__ __forceinline__ double sqrt_(double a) { return sqrt(a); }
 // type as they are (populations, or deviations d_i = f_i - c_i where kDev);
 // load/store (and load64/store64 for FP64 companions) take the reference c_i of
 // population i and convert to and from populations f_i.  The step kernels load
-// with step_in and store with step_out, which give the values the collision
-// works on: the deviations themselves where kDevCollide (FP32 deviations, so that
-// no rounding happens at the scale of w_i), populations otherwise (the 16-bit
-// storages, whose quantisation to 11 or 8 significant bits dwarfs the FP32
-// rounding of f).
+// with raw, hand the stored values to collide_stored and store with pack: the
+// collision works on the deviations themselves where kDevCollide (FP32 deviations,
+// so that no rounding happens at the scale of w_i), and on populations formed from
+// them otherwise (the 16-bit storages, whose quantisation to 11 or 8 significant
+// bits dwarfs the FP32 rounding of f).
 // ---------------------------------------------------------------------------
 struct StoreF64 {
     using S = double;
@@ -222,21 +221,6 @@ struct StoreBF16Dev {
     __device__ static __forceinline__ S store64(double f, double c) { return __double2bfloat16(f - c); }
 };
 
-// The values a step kernel collides on (see kDevCollide), from the stored element s of
-// population i with reference c, and back.
-template <class ST>
-__device__ __forceinline__ typename ST::T step_in(typename ST::S s, typename ST::T c)
-{
-    if constexpr (ST::kDevCollide || !ST::kDev) return ST::raw(s);
-    else return ST::load(s, c);
-}
-template <class ST>
-__device__ __forceinline__ typename ST::S step_out(typename ST::T v, typename ST::T c)
-{
-    if constexpr (ST::kDevCollide || !ST::kDev) return ST::pack(v);
-    else return ST::store(v, c);
-}
-
 template <class T>
 __device__ __forceinline__ T g_entropy(T y);
 
@@ -251,7 +235,7 @@ __device__ __forceinline__ T quad_root(T a, T b, T c)
 {
     const T q = div_(c, b);
     const T p = div_(a, b);
-    return div_(T(2) * q, T(1) + sqrt_(T(1) - T(4) * p * q));
+    return div_(T(2) * q, T(1) + sqrt_(fma(T(-4) * p, q, T(1))));
 }
 
 // ---------------------------------------------------------------------------
@@ -716,6 +700,8 @@ __device__ __forceinline__ float node_collide_pairs(PA &pa, float2 (&xp)[Pairs<D
         // solving here: a warp whose lanes straddle a threshold runs the longer form
         // on all of them instead of each form in turn (the forms agree below FP32
         // rounding, so which one a lane gets moves its path length by less than that).
+        // The scalar tail (sums to path length) spells its fused multiply-adds out, so that every
+        // kernel this is inlined into rounds alike.
         constexpr float kSeriesX = 0.04f, kShortX = 0.005f;
         const int form = __reduce_max_sync(__activemask(), xabs < kShortX ? 0 : (xabs < kSeriesX ? 1 : 2));
         const bool series = form < 2;
@@ -724,52 +710,53 @@ __device__ __forceinline__ float node_collide_pairs(PA &pa, float2 (&xp)[Pairs<D
             float2 M2 = f2(0.0f), M3 = f2(0.0f), M4 = f2(0.0f), S3 = f2(0.0f), S4 = f2(0.0f);
 #pragma unroll
             for (int k = 0; k < NP; ++k) {
-                const float2 xi = xp[k];
-                const float2 fx2 = pmul(fagain(k), pmul(xi, xi)); // f x^2
-                const float2 q3 = pmul(fx2, xi);
-                M2 = padd(M2, fx2);
-                M3 = padd(M3, q3);
-                M4 = pfma(q3, xi, M4);
+                const float2 xi = xp[k], x2 = pmul(xi, xi);
+                const float2 g2 = pmul(fagain(k), x2); // f x^2
+                M2 = padd(M2, g2);
+                M3 = pfma(g2, xi, M3);
+                M4 = pfma(g2, x2, M4);
                 const float2 xm = f2(fminf(xi.x, 0.0f), fminf(xi.y, 0.0f));
-                const float2 q = pmul(fx2, xm); // f x^3 on Omega-, 0 elsewhere
+                const float2 q = pmul(g2, xm); // f x^3 on Omega-, 0 elsewhere
                 S3 = padd(S3, q);
                 S4 = pfma(q, xm, S4);
             }
             const float m2 = M2.x + M2.y;
             m3 = M3.x + M3.y, m4 = M4.x + M4.y;
             sb1 = 0.5f * m2;
-            sc1 = m2 + (m3 * -0.5f + m4 * 0.25f);
-            sc = m2 + (m3 * -0.5f + m4 * (1.0f / 3.0f));
+            sc1 = m2 + fmaf(m3, -0.5f, m4 * 0.25f);
+            sc = m2 + fmaf(m3, -0.5f, m4 * (1.0f / 3.0f));
             s3 = S3.x + S3.y, s4 = S4.x + S4.y;
         } else if (series) {
+            // Omega- through |x|: with A_k = <f, x^(k-1) |x|>, S_k = (M_k - A_k) / 2 for odd
+            // k, and A_k = <f, x^(k-2) x |x|> gives the same for even k.  M_k and A_k share
+            // the products g2 = f x^2, g4 = f x^4 and x |x|, so the nine sums take 13 paired
+            // operations instead of the 16 of separate powers of min(x, 0); the halves add
+            // numbers of the size of S_k itself, so nothing is lost to cancellation.
             float2 M2 = f2(0.0f), M3 = f2(0.0f), M4 = f2(0.0f), M5 = f2(0.0f), M6 = f2(0.0f);
-            float2 S3 = f2(0.0f), S4 = f2(0.0f), S5 = f2(0.0f), S6 = f2(0.0f);
+            float2 A3 = f2(0.0f), A4 = f2(0.0f), A5 = f2(0.0f), A6 = f2(0.0f);
 #pragma unroll
             for (int k = 0; k < NP; ++k) {
-                const float2 xi = xp[k];
-                const float2 x2 = pmul(xi, xi);
-                const float2 fx2 = pmul(fagain(k), x2); // f x^2
-                const float2 q3 = pmul(fx2, xi);
-                const float2 q5 = pmul(q3, x2);
-                M2 = padd(M2, fx2);
-                M3 = padd(M3, q3);
-                M4 = pfma(q3, xi, M4);
-                M5 = padd(M5, q5);
-                M6 = pfma(q5, xi, M6);
-                const float2 xm = f2(fminf(xi.x, 0.0f), fminf(xi.y, 0.0f));
-                const float2 q = pmul(fx2, xm); // f x^3 on Omega-, 0 elsewhere
-                const float2 xm2 = pmul(xm, xm);
-                S3 = padd(S3, q);
-                S4 = pfma(q, xm, S4);
-                S5 = pfma(q, xm2, S5);
-                S6 = pfma(pmul(q, xm), xm2, S6);
+                const float2 xi = xp[k], x2 = pmul(xi, xi);
+                const float2 g2 = pmul(fagain(k), x2); // f x^2
+                const float2 g4 = pmul(g2, x2);        // f x^4
+                const float2 ax = f2(fabsf(xi.x), fabsf(xi.y)), xax = pmul(xi, ax);
+                M2 = padd(M2, g2);
+                M3 = pfma(g2, xi, M3);
+                M4 = padd(M4, g4);
+                M5 = pfma(g4, xi, M5);
+                M6 = pfma(g4, x2, M6);
+                A3 = pfma(g2, ax, A3);
+                A4 = pfma(g2, xax, A4);
+                A5 = pfma(g4, ax, A5);
+                A6 = pfma(g4, xax, A6);
             }
             const float m2 = M2.x + M2.y;
             m3 = M3.x + M3.y, m4 = M4.x + M4.y, m5 = M5.x + M5.y, m6 = M6.x + M6.y;
             sb1 = 0.5f * m2;
-            sc1 = m2 + (m3 * -0.5f + (m4 * 0.25f + (m5 * -0.125f + m6 * 0.0625f))); // <f, 2x^2/(2+x)>
-            sc = m2 + (m3 * -0.5f + (m4 * (1.0f / 3.0f) + (m5 * -0.25f + m6 * 0.2f)));
-            s3 = S3.x + S3.y, s4 = S4.x + S4.y, s5 = S5.x + S5.y, s6 = S6.x + S6.y;
+            sc1 = m2 + fmaf(m3, -0.5f, fmaf(m4, 0.25f, fmaf(m5, -0.125f, m6 * 0.0625f))); // <f, 2x^2/(2+x)>
+            sc = m2 + fmaf(m3, -0.5f, fmaf(m4, 1.0f / 3.0f, fmaf(m5, -0.25f, m6 * 0.2f)));
+            s3 = 0.5f * (m3 - (A3.x + A3.y)), s4 = 0.5f * (m4 - (A4.x + A4.y));
+            s5 = 0.5f * (m5 - (A5.x + A5.y)), s6 = 0.5f * (m6 - (A6.x + A6.y));
         } else {
             float2 b1 = f2(0.0f), c1 = f2(0.0f), c = f2(0.0f);
             float2 S3 = f2(0.0f), S4 = f2(0.0f), S5 = f2(0.0f), S6 = f2(0.0f);
@@ -803,7 +790,7 @@ __device__ __forceinline__ float node_collide_pairs(PA &pa, float2 (&xp)[Pairs<D
                 float bsum;
                 if (series) {
                     const float p3 = m3 - s3, p4 = m4 - s4, p5 = m5 - s5, p6 = m6 - s6;
-                    bsum = 1.25f * p3 + kk * (-0.625f * p4 + kk * (0.375f * p5 + kk * (-0.25f * p6)));
+                    bsum = fmaf(kk, fmaf(kk, fmaf(kk, -0.25f * p6, 0.375f * p5), -0.625f * p4), 1.25f * p3);
                 } else {
                     float2 bp = f2(0.0f);
 #pragma unroll
@@ -818,12 +805,12 @@ __device__ __forceinline__ float node_collide_pairs(PA &pa, float2 (&xp)[Pairs<D
                     }
                     bsum = bp.x + bp.y;
                 }
-                const float b = sb1 - (2.0f / 15.0f) * aL * beta * beta * bsum;
-                const float h = quad_root(beta * beta * s3 * (1.0f / 6.0f), b, sc);
+                const float bb = beta * beta, b = fmaf(-(2.0f / 15.0f) * bb * aL, bsum, sb1);
+                const float h = quad_root(bb * (1.0f / 6.0f) * s3, b, sc);
                 const float hb = h * beta;
-                const float a = beta * beta *
-                                (s3 * (1.0f / 6.0f) - hb * s4 * (1.0f / 12.0f) + hb * hb * s5 * (1.0f / 20.0f) -
-                                 hb * hb * hb * s6 * (1.0f / 5.0f));
+                // a = beta^2 (S3/6 - hb S4/12 + hb^2 S5/20 - hb^3 S6/5), Horner in hb
+                const float a = bb * fmaf(hb, fmaf(hb, fmaf(hb, -0.2f * s6, 0.05f * s5), (-1.0f / 12.0f) * s4),
+                                          (1.0f / 6.0f) * s3);
                 alpha = quad_root(a, b, sc); // alpha_Higher
             }
             br = kBranchSolved;
@@ -847,61 +834,62 @@ __device__ __forceinline__ float node_collide_pairs(PA &pa, float2 (&xp)[Pairs<D
 }
 
 // ---------------------------------------------------------------------------
-// One node's collision on scalar arrays, whatever the compute type: FP32 goes
-// through the packed-pair routine (on deviations d_i = f_i - k_i R when kDev),
-// FP64 through node_collide.  f holds populations (or deviations when kDev) and
-// receives the post-collision values of the same kind.
+// One node's collision on the values v that a step kernel loads (ST::raw: populations,
+// or deviations d_i = f_i - k_i R), whatever the compute type: FP32 goes through the
+// packed-pair routine, FP64 through node_collide.  v receives the post-collision values of
+// the same kind, for ST::pack.  The 16-bit storages turn deviations into populations and
+// back on the packed pairs: 28 paired additions per D3Q27 node instead of 54 scalar ones.
 // ---------------------------------------------------------------------------
-template <int D, class T, bool kRelax = true, bool kDev = false>
-__device__ __forceinline__ T collide(T (&f)[Lattice<D>::Q], T (&x)[Lattice<D>::Q], const CollideParams &p,
-                                     int *branch)
-{
-    constexpr int Q = Lattice<D>::Q;
-    if constexpr (sizeof(T) == 4) {
-        if (p.mode == kModeIterate1) {
-            // alpha_Iterate1 (a comparison variant with logarithms) stays on the scalar
-            // path, which takes populations
-            if constexpr (kDev) {
-#pragma unroll
-                for (int i = 0; i < Q; ++i) f[i] += dev_ref<D, T>(i, p.dunit_f);
-            }
-            const T alpha = node_collide<D, T, kRelax>(f, x, p, branch);
-            if constexpr (kDev) {
-#pragma unroll
-                for (int i = 0; i < Q; ++i) f[i] -= dev_ref<D, T>(i, p.dunit_f);
-            }
-            return alpha;
-        }
-        constexpr int NP = Pairs<D>::NP;
-        float2 fp[NP], xp[NP];
-#pragma unroll
-        for (int k = 0; k < NP; ++k) {
-            const int i1 = pair_pop(D, k, 1);
-            fp[k] = make_float2(f[pair_pop(D, k, 0)], i1 >= 0 ? f[i1] : 1.0f);
-        }
-        PairRegs<NP> pr{fp};
-        const float alpha = node_collide_pairs<D, kRelax, kDev>(pr, xp, p, branch);
-#pragma unroll
-        for (int i = 0; i < Q; ++i) {
-            const int sl = pair_slot(D, i);
-            x[i] = (sl & 1) ? xp[sl >> 1].y : xp[sl >> 1].x;
-            if (kRelax) f[i] = (sl & 1) ? fp[sl >> 1].y : fp[sl >> 1].x;
-        }
-        return alpha;
-    } else {
-        static_assert(!kDev, "deviation storage computes in FP32");
-        return node_collide<D, T, kRelax>(f, x, p, branch);
-    }
-}
-
-// The collision of a step kernel on the values it loaded with step_in: deviations for
-// the FP32 deviation storage, populations otherwise; they are stored back with step_out.
 template <int D, class ST, bool kRelax = true>
 __device__ __forceinline__ typename ST::T collide_stored(typename ST::T (&v)[Lattice<D>::Q],
                                                          typename ST::T (&x)[Lattice<D>::Q],
                                                          const CollideParams &p, int *branch)
 {
-    return collide<D, typename ST::T, kRelax, ST::kDevCollide>(v, x, p, branch);
+    using T = typename ST::T;
+    constexpr int Q = Lattice<D>::Q;
+    if constexpr (sizeof(T) == 4) {
+        if (p.mode == kModeIterate1) {
+            // alpha_Iterate1 (a comparison variant with logarithms) stays on the scalar
+            // path, which takes populations
+            if constexpr (ST::kDev) {
+#pragma unroll
+                for (int i = 0; i < Q; ++i) v[i] += dev_ref<D, T>(i, p.dunit_f);
+            }
+            const T alpha = node_collide<D, T, kRelax>(v, x, p, branch);
+            if constexpr (ST::kDev) {
+#pragma unroll
+                for (int i = 0; i < Q; ++i) v[i] -= dev_ref<D, T>(i, p.dunit_f);
+            }
+            return alpha;
+        }
+        constexpr int NP = Pairs<D>::NP;
+        constexpr bool kConvert = ST::kDev && !ST::kDevCollide;
+        float2 fp[NP], xp[NP];
+        // c_i of pair k (0 in the padding lane, which holds 1)
+        auto ref = [&](int k) { return pmul(f2(kpair<D>(k, 0), kpair<D>(k, 1)), f2(p.dunit_f)); };
+#pragma unroll
+        for (int k = 0; k < NP; ++k) {
+            const int i1 = pair_pop(D, k, 1);
+            fp[k] = make_float2(v[pair_pop(D, k, 0)], i1 >= 0 ? v[i1] : 1.0f);
+            if constexpr (kConvert) fp[k] = padd(fp[k], ref(k));
+        }
+        PairRegs<NP> pr{fp};
+        const float alpha = node_collide_pairs<D, kRelax, ST::kDevCollide>(pr, xp, p, branch);
+        if constexpr (kConvert && kRelax) {
+#pragma unroll
+            for (int k = 0; k < NP; ++k) fp[k] = psub(fp[k], ref(k));
+        }
+#pragma unroll
+        for (int i = 0; i < Q; ++i) {
+            const int sl = pair_slot(D, i);
+            x[i] = (sl & 1) ? xp[sl >> 1].y : xp[sl >> 1].x;
+            if (kRelax) v[i] = (sl & 1) ? fp[sl >> 1].y : fp[sl >> 1].x;
+        }
+        return alpha;
+    } else {
+        static_assert(!ST::kDev, "deviation storage computes in FP32");
+        return node_collide<D, T, kRelax>(v, x, p, branch);
+    }
 }
 
 // ---------------------------------------------------------------------------
@@ -1033,14 +1021,13 @@ __device__ __forceinline__ float2 node_collide_x2(float2 (&f)[9], float2 (&x)[9]
             float2 M2 = f2(0.0f), S3 = f2(0.0f), S4 = f2(0.0f);
 #pragma unroll
             for (int i = 0; i < Q; ++i) {
-                const float2 xi = x[i];
-                const float2 fx2 = pmul(fagain(i), pmul(xi, xi));
-                const float2 q3 = pmul(fx2, xi);
-                M2 = padd(M2, fx2);
-                m3 = padd(m3, q3);
-                m4 = pfma(q3, xi, m4);
+                const float2 xi = x[i], x2 = pmul(xi, xi);
+                const float2 g2 = pmul(fagain(i), x2);
+                M2 = padd(M2, g2);
+                m3 = pfma(g2, xi, m3);
+                m4 = pfma(g2, x2, m4);
                 const float2 xm = f2(fminf(xi.x, 0.0f), fminf(xi.y, 0.0f));
-                const float2 q = pmul(fx2, xm);
+                const float2 q = pmul(g2, xm);
                 S3 = padd(S3, q);
                 S4 = pfma(q, xm, S4);
             }
@@ -1049,32 +1036,30 @@ __device__ __forceinline__ float2 node_collide_x2(float2 (&f)[9], float2 (&x)[9]
             sc = padd(M2, pfma(m3, f2(-0.5f), pmul(m4, f2(1.0f / 3.0f))));
             s3 = S3, s4 = S4;
         } else if (series) {
-            float2 M2 = f2(0.0f), S3 = f2(0.0f), S4 = f2(0.0f), S5 = f2(0.0f), S6 = f2(0.0f);
+            // Omega- sums through |x| (node_collide_pairs)
+            float2 M2 = f2(0.0f), A3 = f2(0.0f), A4 = f2(0.0f), A5 = f2(0.0f), A6 = f2(0.0f);
 #pragma unroll
             for (int i = 0; i < Q; ++i) {
-                const float2 xi = x[i];
-                const float2 x2 = pmul(xi, xi);
-                const float2 fx2 = pmul(fagain(i), x2);
-                const float2 q3 = pmul(fx2, xi);
-                const float2 q5 = pmul(q3, x2);
-                M2 = padd(M2, fx2);
-                m3 = padd(m3, q3);
-                m4 = pfma(q3, xi, m4);
-                m5 = padd(m5, q5);
-                m6 = pfma(q5, xi, m6);
-                const float2 xm = f2(fminf(xi.x, 0.0f), fminf(xi.y, 0.0f));
-                const float2 q = pmul(fx2, xm);
-                const float2 xm2 = pmul(xm, xm);
-                S3 = padd(S3, q);
-                S4 = pfma(q, xm, S4);
-                S5 = pfma(q, xm2, S5);
-                S6 = pfma(pmul(q, xm), xm2, S6);
+                const float2 xi = x[i], x2 = pmul(xi, xi);
+                const float2 g2 = pmul(fagain(i), x2);
+                const float2 g4 = pmul(g2, x2);
+                const float2 ax = f2(fabsf(xi.x), fabsf(xi.y)), xax = pmul(xi, ax);
+                M2 = padd(M2, g2);
+                m3 = pfma(g2, xi, m3);
+                m4 = padd(m4, g4);
+                m5 = pfma(g4, xi, m5);
+                m6 = pfma(g4, x2, m6);
+                A3 = pfma(g2, ax, A3);
+                A4 = pfma(g2, xax, A4);
+                A5 = pfma(g4, ax, A5);
+                A6 = pfma(g4, xax, A6);
             }
             sb1 = pmul(f2(0.5f), M2);
             // <f, 2x^2/(2+x)> and c, Horner in the power sums
             sc1 = padd(M2, pfma(m3, f2(-0.5f), pfma(m4, f2(0.25f), pfma(m5, f2(-0.125f), pmul(m6, f2(0.0625f))))));
             sc = padd(M2, pfma(m3, f2(-0.5f), pfma(m4, f2(1.0f / 3.0f), pfma(m5, f2(-0.25f), pmul(m6, f2(0.2f))))));
-            s3 = S3, s4 = S4, s5 = S5, s6 = S6;
+            s3 = pmul(f2(0.5f), psub(m3, A3)), s4 = pmul(f2(0.5f), psub(m4, A4));
+            s5 = pmul(f2(0.5f), psub(m5, A5)), s6 = pmul(f2(0.5f), psub(m6, A6));
         } else {
             float2 b1 = f2(0.0f), c1 = f2(0.0f), c = f2(0.0f), S3 = f2(0.0f), S4 = f2(0.0f), S5 = f2(0.0f),
                    S6 = f2(0.0f);
@@ -1172,8 +1157,7 @@ __host__ __device__ constexpr int nodes_per_thread()
     return (D == 2 && sizeof(typename ST::T) == 4) ? 2 : 1;
 }
 
-// Two nodes' collision in a step kernel, on the values loaded with step_in (as
-// collide_stored): node_collide_x2 where nodes_per_thread is 2 (alpha_Iterate1, a
+// Two nodes' collision in a step kernel, on the stored values (as collide_stored): node_collide_x2 where nodes_per_thread is 2 (alpha_Iterate1, a
 // comparison variant with logarithms, stays on the one-node path), else node by node.
 template <int D, class ST, bool kRelax = true>
 __device__ __forceinline__ void collide2_stored(typename ST::T (&fa)[Lattice<D>::Q],
@@ -1183,13 +1167,18 @@ __device__ __forceinline__ void collide2_stored(typename ST::T (&fa)[Lattice<D>:
     constexpr int Q = Lattice<D>::Q;
     if constexpr (nodes_per_thread<D, ST>() == 2) {
         if (p.mode != kModeIterate1) {
+            constexpr bool kConvert = ST::kDev && !ST::kDevCollide;
             float2 v[9], x[9];
             int br[2];
 #pragma unroll
-            for (int i = 0; i < 9; ++i) v[i] = make_float2(fa[i], fb[i]);
+            for (int i = 0; i < 9; ++i) {
+                v[i] = make_float2(fa[i], fb[i]);
+                if constexpr (kConvert) v[i] = padd(v[i], f2(dev_ref<2, float>(i, p.dunit_f)));
+            }
             node_collide_x2<kRelax, ST::kDevCollide>(v, x, p, br);
 #pragma unroll
             for (int i = 0; i < 9; ++i) {
+                if constexpr (kConvert) v[i] = psub(v[i], f2(dev_ref<2, float>(i, p.dunit_f)));
                 fa[i] = v[i].x;
                 fb[i] = v[i].y;
             }
@@ -1202,13 +1191,13 @@ __device__ __forceinline__ void collide2_stored(typename ST::T (&fa)[Lattice<D>:
     collide_stored<D, ST, kRelax>(fb, x, p, &br);
 }
 
-// Population loads of the step kernels: through the read-only path (ld.global.nc), or,
-// with kStream, with the evict-first (streaming) policy (ld.global.cs): each line is read
-// once from DRAM and again, within a few warps, by the neighbours' shifted loads.  The
-// D3Q27 step takes the second where most nodes need the longer coefficient forms: there it
-// spills through L1, and population lines that leave L1 first keep room for the spills
-// (D3Q27 256^3 FP32, same box: 0.6807 against 0.6867 ms late in the benchmark flow, but
-// 0.5787 against 0.5727 early, where the step is bound by DRAM).
+// Population loads of the step kernels.  D3Q27 loads with the evict-first (streaming)
+// policy (ld.global.cs): each line comes once from DRAM and is read again, within a few
+// warps, by the neighbours' shifted loads, while the register spills of the collision pass
+// through the same L1; population lines that leave first keep room for them (256^3 FP32
+// Taylor-Green start: 0.543 against 0.552 ms per step through the read-only path; 203 x 150
+// x 131 developed flow: 0.1525 against 0.157).  D2Q9, which does not spill to speak of, loads
+// through the read-only path.
 template <bool kStream, class S>
 __device__ __forceinline__ S ld_pop(const S *p)
 {
@@ -1220,7 +1209,7 @@ __device__ __forceinline__ S ld_pop(const S *p)
 // Pull streaming (Eq. advection): population i at node (x, y, z) comes from
 // (x - c_ix, y - c_iy, z - c_iz) with periodic wrap.
 // ---------------------------------------------------------------------------
-// f receives populations (ST::load); with kStep, the values a step kernel collides on (step_in).
+// f receives populations (ST::load); with kStep, the values a step kernel collides on (ST::raw).
 template <int D, class ST, bool kStep = false>
 __device__ __forceinline__ void pull_load(const typename ST::S *__restrict__ fin, const Geometry &g,
                                           int x, int y, int z, float R,
@@ -1240,7 +1229,7 @@ __device__ __forceinline__ void pull_load(const typename ST::S *__restrict__ fin
         const int sz = cz == 1 ? zm : (cz == -1 ? zp : z);
         const int64_t src = ((int64_t)sz * g.ny + sy) * g.nx + sx;
         const typename ST::S sv = __ldg(fin + (int64_t)i * g.N + src);
-        f[i] = kStep ? step_in<ST>(sv, dev_ref<D, T>(i, R)) : ST::load(sv, dev_ref<D, T>(i, R));
+        f[i] = kStep ? ST::raw(sv) : ST::load(sv, dev_ref<D, T>(i, R));
     }
 }
 

@@ -13,6 +13,8 @@
 //              then shared memory, then one atomic per block and quantity
 #pragma once
 
+#include <type_traits>
+
 #include "elbm_device.cuh"
 #include "elbm_launch.h"
 #include "elbm_tma.cuh"
@@ -48,9 +50,21 @@ __device__ __forceinline__ void node_coords(int64_t n, const Geometry &g, int &x
     y = int(t - (int64_t)z * g.ny);
 }
 
-// One node per thread.  Launched either on a 3D grid (x from blockIdx.x,
-// y = blockIdx.y, z = blockIdx.z: no index arithmetic, 32-bit offsets) or, when
-// ny or nz exceed the grid limits or Q N reaches 2^32, on a 1D grid over all nodes.
+// Addressing of the direct step kernel (template parameter kAddr), chosen by the launcher
+// from the size of the domain:
+//   kAddrBytes  Q N elements fill less than 2^32 bytes: 32-bit byte offsets from the buffer
+//   kAddrElems  Q N < 2^32 elements: 32-bit element offsets, scaled by the load and store
+//   kAddrWide   anything else: a 1D grid over all nodes, 64-bit indices
+// One node per thread: blocks of consecutive nodes of an xy-plane (blockIdx.y = z), so that
+// a width that is no multiple of the block leaves no idle warps; x and y come from one
+// multiplication by a precomputed reciprocal (RowDiv).  D3Q27, ms per step, one block row per
+// x-row and element offsets against this: 0.569 and 0.543 (256^3 FP32, Taylor-Green start),
+// 0.185 and 0.1525 (203 x 150 x 131, developed flow; a fifth of the threads of its rows of 256
+// were idle), 0.2125 and 0.165 (176 x 144 x 160, FP16 deviations).  The addresses cost
+// either the multiply-add pipe that the collision needs (a scaled 32-bit offset is one wide
+// multiply-add per access) or two additions on the integer pipe, which is less busy: byte
+// offsets are 0.543 against 0.550 (256^3) and 0.165 against 0.175 (FP16 deviations).  Two
+// nodes per thread (D2Q9): blocks along x-rows, y = blockIdx.y.
 // Minimum resident blocks per SM requested from the register allocator for the
 // direct step kernel.  D3Q27 with FP32 storage: 7 blocks of 128 (72 registers).
 // Near equilibrium the step is bound by load latency, and the extra resident warps
@@ -98,18 +112,36 @@ constexpr int step_threads()
 }
 #define ELBM_STEP_BOUNDS __launch_bounds__(step_threads<ST>(), step_min_blocks<ST>())
 
-template <class ST, bool kGrid3D, bool kForce = false, bool kStream = false>
+enum { kAddrBytes = 0, kAddrElems = 1, kAddrWide = 2 };
+
+// Exact n / d for n < 2^31: (umulhi(magic, n) + n) >> shift with shift = ceil(log2 d) and
+// magic = floor(2^32 (2^shift - d) / d) + 1 (Granlund and Montgomery; the sum stays below
+// 2^32 because magic < 2^32 makes umulhi(magic, n) < n).
+struct RowDiv {
+    uint32_t magic, shift;
+};
+inline RowDiv row_div(uint32_t d)
+{
+    RowDiv r{0, 0};
+    while ((uint64_t(1) << r.shift) < d) ++r.shift;
+    r.magic = uint32_t(((uint64_t(1) << 32) * ((uint64_t(1) << r.shift) - d)) / d + 1);
+    return r;
+}
+__device__ __forceinline__ uint32_t div_row(uint32_t n, RowDiv r) { return (__umulhi(r.magic, n) + n) >> r.shift; }
+
+template <class ST, int kAddr, bool kForce = false>
 __global__ void ELBM_STEP_BOUNDS k_step(const typename ST::S *__restrict__ fin,
                                                     typename ST::S *__restrict__ fout, Geometry g,
-                                                    CollideParams p)
+                                                    CollideParams p, RowDiv rd)
 {
+    using S = typename ST::S;
     using T = typename ST::T;
     if constexpr (nodes_per_thread<D, ST>() == 2) {
         // Two nodes per thread (pair_node); a second node past the end of the row (or of
         // the domain) is a copy of the first, collided and not stored.
         constexpr uint32_t H = kPairSpan / 2;
         T fa[Q], fb[Q];
-        if constexpr (kGrid3D) {
+        if constexpr (kAddr != kAddrWide) {
             const uint32_t nx = uint32_t(g.nx), ny = uint32_t(g.ny), N = uint32_t(g.N);
             const uint32_t xa = blockIdx.x * kStepBlock + pair_node(threadIdx.x);
             if (xa >= nx) return;
@@ -124,22 +156,22 @@ __global__ void ELBM_STEP_BOUNDS k_step(const typename ST::S *__restrict__ fin,
                 return uint32_t(i) * N + sy * nx + sx;
             };
 #pragma unroll
-            for (int i = 0; i < Q; ++i) fa[i] = step_in<ST>(ld_pop<false>(fin + src(xa, i)), dev_ref<D, T>(i, p.dunit_f));
+            for (int i = 0; i < Q; ++i) fa[i] = ST::raw(ld_pop<false>(fin + src(xa, i)));
 #pragma unroll
-            for (int i = 0; i < Q; ++i) fb[i] = step_in<ST>(ld_pop<false>(fin + src(xb, i)), dev_ref<D, T>(i, p.dunit_f));
+            for (int i = 0; i < Q; ++i) fb[i] = ST::raw(ld_pop<false>(fin + src(xb, i)));
             collide2_stored<D, ST, true>(fa, fb, p);
             if constexpr (kForce) {
-                add_force<D, T, ST::kDevCollide>(fa, p);
-                add_force<D, T, ST::kDevCollide>(fb, p);
+                add_force<D, T, ST::kDev>(fa, p);
+                add_force<D, T, ST::kDev>(fb, p);
             }
             const uint32_t na = y * nx + xa, nb = y * nx + xb;
 #pragma unroll
             for (int i = 0; i < Q; ++i)
-                __stcs(fout + (uint32_t(i) * N + na), step_out<ST>(fa[i], dev_ref<D, T>(i, p.dunit_f)));
+                __stcs(fout + (uint32_t(i) * N + na), ST::pack(fa[i]));
             if (hasb) {
 #pragma unroll
                 for (int i = 0; i < Q; ++i)
-                    __stcs(fout + (uint32_t(i) * N + nb), step_out<ST>(fb[i], dev_ref<D, T>(i, p.dunit_f)));
+                    __stcs(fout + (uint32_t(i) * N + nb), ST::pack(fb[i]));
             }
         } else {
             const int64_t na = (int64_t)blockIdx.x * kStepBlock + pair_node(threadIdx.x);
@@ -153,47 +185,53 @@ __global__ void ELBM_STEP_BOUNDS k_step(const typename ST::S *__restrict__ fin,
             pull_load<D, ST, true>(fin, g, x, y, z, p.dunit_f, fb);
             collide2_stored<D, ST, true>(fa, fb, p);
             if constexpr (kForce) {
-                add_force<D, T, ST::kDevCollide>(fa, p);
-                add_force<D, T, ST::kDevCollide>(fb, p);
+                add_force<D, T, ST::kDev>(fa, p);
+                add_force<D, T, ST::kDev>(fb, p);
             }
 #pragma unroll
-            for (int i = 0; i < Q; ++i) __stcs(fout + (int64_t)i * g.N + na, step_out<ST>(fa[i], dev_ref<D, T>(i, p.dunit_f)));
+            for (int i = 0; i < Q; ++i) __stcs(fout + (int64_t)i * g.N + na, ST::pack(fa[i]));
             if (hasb) {
 #pragma unroll
                 for (int i = 0; i < Q; ++i)
-                    __stcs(fout + (int64_t)i * g.N + nb, step_out<ST>(fb[i], dev_ref<D, T>(i, p.dunit_f)));
+                    __stcs(fout + (int64_t)i * g.N + nb, ST::pack(fb[i]));
             }
         }
         return;
     }
     T f[Q], xd[Q]; // the stored values (deviations for deviation storage)
     int br;
-    if constexpr (kGrid3D) {
-        // 3D grid with Q N < 2^32: element offsets in 32 bits (the source rows of
-        // (y - c_y, z - c_z) depend on the block only).  Measured faster on GB300 than
-        // per-thread base pointers with block-uniform row offsets.
-        const uint32_t x = blockIdx.x * kStepBlock + threadIdx.x;
+    if constexpr (kAddr != kAddrWide) {
         const uint32_t nx = uint32_t(g.nx), ny = uint32_t(g.ny), nz = uint32_t(g.nz), N = uint32_t(g.N);
-        if (x >= nx) return;
-        const uint32_t y = blockIdx.y, z = blockIdx.z;
-        const uint32_t xm = x == 0 ? nx - 1 : x - 1, xp = x == nx - 1 ? 0 : x + 1;
-        const uint32_t ym = y == 0 ? ny - 1 : y - 1, yp = y == ny - 1 ? 0 : y + 1;
-        const uint32_t zm = z == 0 ? nz - 1 : z - 1, zp = z == nz - 1 ? 0 : z + 1;
-        // element offset of population i pulled into this node
-        auto src = [&](int i) -> uint32_t {
-            const int cx = vel(D, i, 0), cy = vel(D, i, 1), cz = D == 3 ? vel(D, i, 2) : 0;
-            const uint32_t sx = cx == 1 ? xm : (cx == -1 ? xp : x);
-            const uint32_t sy = cy == 1 ? ym : (cy == -1 ? yp : y);
-            const uint32_t sz = cz == 1 ? zm : (cz == -1 ? zp : z);
-            return uint32_t(i) * N + (sz * ny + sy) * nx + sx;
+        const uint32_t plane = nx * ny, xy = blockIdx.x * kStepBlock + threadIdx.x, z = blockIdx.y;
+        if (xy >= plane) return;
+        const uint32_t y = div_row(xy, rd), x = xy - y * nx;
+        // offsets of the nine (c_x, c_y) sources in a plane; the rest of an address is the
+        // same for the whole block
+        constexpr uint32_t B = kAddr == kAddrBytes ? uint32_t(sizeof(S)) : 1u;
+        const uint32_t sx[3] = {x == nx - 1 ? 0 : x + 1, x, x == 0 ? nx - 1 : x - 1};
+        const uint32_t sy[3] = {y == ny - 1 ? 0 : (y + 1) * nx, y * nx, (y == 0 ? ny - 1 : y - 1) * nx};
+        const uint32_t sz[3] = {z == nz - 1 ? 0 : z + 1, z, z == 0 ? nz - 1 : z - 1};
+        auto at = [](auto *base, uint32_t o) {
+            using P = decltype(base);
+            if constexpr (kAddr == kAddrBytes) {
+                using C = std::conditional_t<std::is_const_v<std::remove_pointer_t<P>>, const char, char>;
+                return reinterpret_cast<P>(reinterpret_cast<C *>(base) + o);
+            } else {
+                return base + o;
+            }
         };
 #pragma unroll
-        for (int i = 0; i < Q; ++i) f[i] = step_in<ST>(ld_pop<kStream>(fin + src(i)), dev_ref<D, T>(i, p.dunit_f));
+        for (int i = 0; i < Q; ++i) {
+            const int cx = vel(D, i, 0), cy = vel(D, i, 1), cz = D == 3 ? vel(D, i, 2) : 0;
+            const uint32_t o = (sy[cy + 1] + sx[cx + 1]) * B;
+            const uint32_t b = (uint32_t(i) * N + sz[cz + 1] * plane) * B;
+            f[i] = ST::raw(ld_pop<D == 3>(at(fin, o + b)));
+        }
         collide_stored<D, ST, true>(f, xd, p, &br);
-        if constexpr (kForce) add_force<D, T, ST::kDevCollide>(f, p);
-        const uint32_t n = (z * ny + y) * nx + x;
+        if constexpr (kForce) add_force<D, T, ST::kDev>(f, p);
+        const uint32_t n = (z * plane + xy) * B;
 #pragma unroll
-        for (int i = 0; i < Q; ++i) __stcs(fout + (uint32_t(i) * N + n), step_out<ST>(f[i], dev_ref<D, T>(i, p.dunit_f)));
+        for (int i = 0; i < Q; ++i) __stcs(at(fout, uint32_t(i) * N * B + n), ST::pack(f[i]));
     } else {
         const int64_t n = (int64_t)blockIdx.x * kStepBlock + threadIdx.x;
         if (n >= g.N) return;
@@ -201,9 +239,9 @@ __global__ void ELBM_STEP_BOUNDS k_step(const typename ST::S *__restrict__ fin,
         node_coords(n, g, x, y, z);
         pull_load<D, ST, true>(fin, g, x, y, z, p.dunit_f, f);
         collide_stored<D, ST, true>(f, xd, p, &br);
-        if constexpr (kForce) add_force<D, T, ST::kDevCollide>(f, p);
+        if constexpr (kForce) add_force<D, T, ST::kDev>(f, p);
 #pragma unroll
-        for (int i = 0; i < Q; ++i) __stcs(fout + (int64_t)i * g.N + n, step_out<ST>(f[i], dev_ref<D, T>(i, p.dunit_f)));
+        for (int i = 0; i < Q; ++i) __stcs(fout + (int64_t)i * g.N + n, ST::pack(f[i]));
     }
 }
 
@@ -692,7 +730,7 @@ __global__ void __launch_bounds__(kAuxBlock) k_diag(const typename ST::S *__rest
         T f[Q], xd[Q], fc[Q];
         pull_load<D, ST, true>(fin, g, x, y, z, p.dunit_f, f); // stored values, as the step collides them
 #pragma unroll
-        for (int i = 0; i < Q; ++i) fc[i] = ST::kDevCollide ? f[i] + dev_ref<D, T>(i, p.dunit_f) : f[i]; // populations
+        for (int i = 0; i < Q; ++i) fc[i] = ST::kDev ? f[i] + dev_ref<D, T>(i, p.dunit_f) : f[i]; // populations
         int br;
         const T alpha_t = collide_stored<D, ST, false>(f, xd, p, &br);
         dt.node(fc, xd, alpha_t, br, p, s_hist);
@@ -742,15 +780,15 @@ __global__ void __launch_bounds__(kStepBlock, step_diag_min_blocks<ST>()) k_step
         };
 #pragma unroll
         for (int i = 0; i < Q; ++i) {
-            f[i] = step_in<ST>(ld_pop<false>(fin + src(i)), dev_ref<D, T>(i, p.dunit_f));
-            fc[i] = ST::kDevCollide ? f[i] + dev_ref<D, T>(i, p.dunit_f) : f[i]; // populations
+            f[i] = ST::raw(ld_pop<false>(fin + src(i)));
+            fc[i] = ST::kDev ? f[i] + dev_ref<D, T>(i, p.dunit_f) : f[i]; // populations
         }
         int br;
         const T alpha_t = collide_stored<D, ST, true>(f, xd, p, &br);
         dt.node(fc, xd, alpha_t, br, p, s_hist);
         const uint32_t n = (z * ny + y) * nx + x;
 #pragma unroll
-        for (int i = 0; i < Q; ++i) __stcs(fout + (uint32_t(i) * N + n), step_out<ST>(f[i], dev_ref<D, T>(i, p.dunit_f)));
+        for (int i = 0; i < Q; ++i) __stcs(fout + (uint32_t(i) * N + n), ST::pack(f[i]));
     }
     diag_finish<kStepBlock>(dt, acc, s_hist);
 }
@@ -777,21 +815,21 @@ __device__ __forceinline__ void step2_row(const typename ST::S *in, typename ST:
     auto ld = [&](uint32_t o) { return kCoherent ? in[o] : ld_pop<false>(in + o); };
     T fa[Q], fb[Q];
 #pragma unroll
-    for (int i = 0; i < Q; ++i) fa[i] = step_in<ST>(ld(src(xa, i)), dev_ref<D, T>(i, p.dunit_f));
+    for (int i = 0; i < Q; ++i) fa[i] = ST::raw(ld(src(xa, i)));
 #pragma unroll
-    for (int i = 0; i < Q; ++i) fb[i] = step_in<ST>(ld(src(xb, i)), dev_ref<D, T>(i, p.dunit_f));
+    for (int i = 0; i < Q; ++i) fb[i] = ST::raw(ld(src(xb, i)));
     collide2_stored<D, ST, true>(fa, fb, p);
     const uint32_t na = y * nx + xa, nb = y * nx + xb;
 #pragma unroll
     for (int i = 0; i < Q; ++i) {
-        const typename ST::S v = step_out<ST>(fa[i], dev_ref<D, T>(i, p.dunit_f));
+        const typename ST::S v = ST::pack(fa[i]);
         if (kCoherent) out[uint32_t(i) * N + na] = v;
         else __stcs(out + (uint32_t(i) * N + na), v);
     }
     if (hasb) {
 #pragma unroll
         for (int i = 0; i < Q; ++i) {
-            const typename ST::S v = step_out<ST>(fb[i], dev_ref<D, T>(i, p.dunit_f));
+            const typename ST::S v = ST::pack(fb[i]);
             if (kCoherent) out[uint32_t(i) * N + nb] = v;
             else __stcs(out + (uint32_t(i) * N + nb), v);
         }
@@ -865,12 +903,12 @@ __global__ void __launch_bounds__(BX / nodes_per_thread<D, ST>(), batch_min_bloc
         return uint32_t(i) * N + (sz * ny + sy) * nx + sx;
     };
 #pragma unroll
-    for (int i = 0; i < Q; ++i) f[i] = step_in<ST>(ld_pop<false>(in + src(i)), dev_ref<D, T>(i, p.dunit_f));
+    for (int i = 0; i < Q; ++i) f[i] = ST::raw(ld_pop<false>(in + src(i)));
     int br;
     collide_stored<D, ST, true>(f, xd, p, &br);
     const uint32_t n = (z * ny + y) * nx + x;
 #pragma unroll
-    for (int i = 0; i < Q; ++i) __stcs(out + (uint32_t(i) * N + n), step_out<ST>(f[i], dev_ref<D, T>(i, p.dunit_f)));
+    for (int i = 0; i < Q; ++i) __stcs(out + (uint32_t(i) * N + n), ST::pack(f[i]));
 }
 
 // --------------------------------------------------------------------------
@@ -970,12 +1008,12 @@ __global__ void __launch_bounds__(BX / nodes_per_thread<D, ST>()) k_step_persist
                 return uint32_t(i) * N + (sz * ny + sy) * nx + sx;
             };
 #pragma unroll
-            for (int i = 0; i < Q; ++i) f[i] = step_in<ST>(in[src(i)], dev_ref<D, T>(i, p.dunit_f));
+            for (int i = 0; i < Q; ++i) f[i] = ST::raw(in[src(i)]);
             int br;
             collide_stored<D, ST, true>(f, xd, p, &br);
             const uint32_t n = (z * ny + y) * nx + x;
 #pragma unroll
-            for (int i = 0; i < Q; ++i) out[uint32_t(i) * N + n] = step_out<ST>(f[i], dev_ref<D, T>(i, p.dunit_f));
+            for (int i = 0; i < Q; ++i) out[uint32_t(i) * N + n] = ST::pack(f[i]);
         }
         __syncthreads(); // every store of this chunk issued; s_ticket and s_ok read by all
         if (threadIdx.x == 0) {
@@ -1237,47 +1275,38 @@ cudaError_t ELBM_CAT(launch_step, ELBM_SUFFIX)(int storage, const void *fin, voi
 #undef ELBM_ROWS_FOR
     }
     if (kernel == ELBM_KERNEL_ROWS) return cudaErrorNotSupported;
-    if (g.ny <= 65535 && g.nz <= 65535 && uint64_t(Q) * uint64_t(g.N) <= 0xffffffffull) {
-        const dim3 grid(unsigned((g.nx + kStepBlock - 1) / kStepBlock), unsigned(g.ny), unsigned(g.nz));
-        if constexpr (D == 3) {
-            // the evict-first variant for the FP32-arithmetic storages (FP64, the parity
-            // path, keeps the read-only path)
-            if (!forced && p.pop_stream && storage != ELBM_STORE_F64) {
-#define ELBM_STREAM_STEP(STT)                                                                     \
-    k_step<STT, true, false, true><<<grid, step_threads<STT>(), 0, s>>>(                          \
-        static_cast<const typename STT::S *>(fin), static_cast<typename STT::S *>(fout), g, p)
-                switch (storage) {
-                case ELBM_STORE_F32: ELBM_STREAM_STEP(StoreF32); break;
-                case ELBM_STORE_F32DEV: ELBM_STREAM_STEP(StoreF32Dev); break;
-                case ELBM_STORE_F16DEV: ELBM_STREAM_STEP(StoreF16Dev); break;
-                case ELBM_STORE_BF16DEV: ELBM_STREAM_STEP(StoreBF16Dev); break;
-                default: return cudaErrorInvalidValue;
-                }
-#undef ELBM_STREAM_STEP
-                return cudaGetLastError();
-            }
-        }
-        if (forced) {
-            ELBM_STORAGE_SWITCH(storage, (k_step<ST, true, true><<<grid, step_threads<ST>(), 0, s>>>(
-                                             static_cast<const typename ST::S *>(fin),
-                                             static_cast<typename ST::S *>(fout), g, p)));
-        } else {
-            ELBM_STORAGE_SWITCH(storage, (k_step<ST, true><<<grid, step_threads<ST>(), 0, s>>>(
-                                             static_cast<const typename ST::S *>(fin),
-                                             static_cast<typename ST::S *>(fout), g, p)));
-        }
+    const uint64_t elems = uint64_t(Q) * uint64_t(g.N);
+    const RowDiv rd = row_div(uint32_t(g.nx));
+#define ELBM_DIRECT_STEP(ADDR, GRID)                                                                   \
+    if (forced) {                                                                                      \
+        ELBM_STORAGE_SWITCH(storage, (k_step<ST, (ADDR == kAddrBytes ? kAddrElems : ADDR), true>       \
+                                      <<<GRID, step_threads<ST>(), 0, s>>>(                            \
+                                          static_cast<const typename ST::S *>(fin),                    \
+                                          static_cast<typename ST::S *>(fout), g, p, rd)));            \
+    } else {                                                                                           \
+        ELBM_STORAGE_SWITCH(storage, (k_step<ST, (nodes_per_thread<D, ST>() == 2 && ADDR == kAddrBytes \
+                                                      ? kAddrElems                                     \
+                                                      : ADDR)><<<GRID, step_threads<ST>(), 0, s>>>(    \
+                                          static_cast<const typename ST::S *>(fin),                    \
+                                          static_cast<typename ST::S *>(fout), g, p, rd)));            \
+    }
+    const bool pair = D == 2 && storage != ELBM_STORE_F64; // two nodes per thread, blocks along rows
+    const int64_t plane = int64_t(g.nx) * g.ny;
+    if (elems > 0xffffffffull || (pair ? g.ny : g.nz) > 65535) {
+        ELBM_DIRECT_STEP(kAddrWide, blocks_for(g.N, kStepBlock))
     } else {
-        if (forced) {
-            ELBM_STORAGE_SWITCH(storage,
-                                (k_step<ST, false, true><<<blocks_for(g.N, kStepBlock), step_threads<ST>(), 0, s>>>(
-                                    static_cast<const typename ST::S *>(fin),
-                                    static_cast<typename ST::S *>(fout), g, p)));
+        const dim3 grid = pair ? dim3(blocks_for(g.nx, kStepBlock), unsigned(g.ny))
+                               : dim3(blocks_for(plane, kStepBlock), unsigned(g.nz));
+        const uint64_t size = storage == ELBM_STORE_F64                                       ? 8
+                              : storage == ELBM_STORE_F32 || storage == ELBM_STORE_F32DEV ? 4
+                                                                                              : 2;
+        if (elems * size <= 0xffffffffull) {
+            ELBM_DIRECT_STEP(kAddrBytes, grid)
         } else {
-            ELBM_STORAGE_SWITCH(storage, (k_step<ST, false><<<blocks_for(g.N, kStepBlock), step_threads<ST>(), 0, s>>>(
-                                             static_cast<const typename ST::S *>(fin),
-                                             static_cast<typename ST::S *>(fout), g, p)));
+            ELBM_DIRECT_STEP(kAddrElems, grid)
         }
     }
+#undef ELBM_DIRECT_STEP
     return cudaGetLastError();
 }
 
