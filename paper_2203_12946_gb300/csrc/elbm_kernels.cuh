@@ -64,7 +64,9 @@ __device__ __forceinline__ void node_coords(int64_t n, const Geometry &g, int &x
 // either the multiply-add pipe that the collision needs (a scaled 32-bit offset is one wide
 // multiply-add per access) or two additions on the integer pipe, which is less busy: byte
 // offsets are 0.543 against 0.550 (256^3) and 0.165 against 0.175 (FP16 deviations).  Two
-// nodes per thread (D2Q9): blocks along x-rows, y = blockIdx.y.
+// nodes per thread (D2Q9): blocks along x-rows, y = blockIdx.y; byte offsets there are 55.8
+// against 59.0 us per step (2048^2 FP32, developed flow) and 24.6 against 26.5 (1501 x 997,
+// FP32 and FP16 deviations), and leave the DRAM-bound shear layers as they were.
 // Minimum resident blocks per SM requested from the register allocator for the
 // direct step kernel.  D3Q27 with FP32 storage: 7 blocks of 128 (72 registers).
 // Near equilibrium the step is bound by load latency, and the extra resident warps
@@ -127,6 +129,14 @@ inline RowDiv row_div(uint32_t d)
     r.magic = uint32_t(((uint64_t(1) << 32) * ((uint64_t(1) << r.shift) - d)) / d + 1);
     return r;
 }
+// Element at offset o of a buffer: o in bytes (kAddrBytes) or elements.
+template <int kAddr, class S>
+__device__ __forceinline__ S *at(S *base, uint32_t o)
+{
+    using C = std::conditional_t<std::is_const_v<S>, const char, char>;
+    if constexpr (kAddr == kAddrBytes) return reinterpret_cast<S *>(reinterpret_cast<C *>(base) + o);
+    else return base + o;
+}
 __device__ __forceinline__ uint32_t div_row(uint32_t n, RowDiv r) { return (__umulhi(r.magic, n) + n) >> r.shift; }
 
 template <class ST, int kAddr, bool kForce = false>
@@ -148,30 +158,26 @@ __global__ void ELBM_STEP_BOUNDS k_step(const typename ST::S *__restrict__ fin,
             const bool hasb = xa + H < nx;
             const uint32_t xb = hasb ? xa + H : xa;
             const uint32_t y = blockIdx.y;
-            const uint32_t ym = y == 0 ? ny - 1 : y - 1, yp = y == ny - 1 ? 0 : y + 1;
-            auto src = [&](uint32_t x, int i) -> uint32_t {
-                const int cx = vel(D, i, 0), cy = vel(D, i, 1);
-                const uint32_t sx = cx == 1 ? (x == 0 ? nx - 1 : x - 1) : (cx == -1 ? (x == nx - 1 ? 0 : x + 1) : x);
-                const uint32_t sy = cy == 1 ? ym : (cy == -1 ? yp : y);
-                return uint32_t(i) * N + sy * nx + sx;
-            };
+            constexpr uint32_t B = kAddr == kAddrBytes ? uint32_t(sizeof(S)) : 1u;
+            const uint32_t ca[3] = {xa == nx - 1 ? 0 : xa + 1, xa, xa == 0 ? nx - 1 : xa - 1};
+            const uint32_t cb[3] = {xb == nx - 1 ? 0 : xb + 1, xb, xb == 0 ? nx - 1 : xb - 1};
+            const uint32_t sy[3] = {y == ny - 1 ? 0 : (y + 1) * nx, y * nx, (y == 0 ? ny - 1 : y - 1) * nx};
+            auto row = [&](int i) { return (uint32_t(i) * N + sy[vel(D, i, 1) + 1]) * B; };
 #pragma unroll
-            for (int i = 0; i < Q; ++i) fa[i] = ST::raw(ld_pop<false>(fin + src(xa, i)));
+            for (int i = 0; i < Q; ++i) fa[i] = ST::raw(ld_pop<false>(at<kAddr>(fin, ca[vel(D, i, 0) + 1] * B + row(i))));
 #pragma unroll
-            for (int i = 0; i < Q; ++i) fb[i] = ST::raw(ld_pop<false>(fin + src(xb, i)));
+            for (int i = 0; i < Q; ++i) fb[i] = ST::raw(ld_pop<false>(at<kAddr>(fin, cb[vel(D, i, 0) + 1] * B + row(i))));
             collide2_stored<D, ST, true>(fa, fb, p);
             if constexpr (kForce) {
                 add_force<D, T, ST::kDev>(fa, p);
                 add_force<D, T, ST::kDev>(fb, p);
             }
-            const uint32_t na = y * nx + xa, nb = y * nx + xb;
+            const uint32_t na = (y * nx + xa) * B, nb = (y * nx + xb) * B;
 #pragma unroll
-            for (int i = 0; i < Q; ++i)
-                __stcs(fout + (uint32_t(i) * N + na), ST::pack(fa[i]));
+            for (int i = 0; i < Q; ++i) __stcs(at<kAddr>(fout, uint32_t(i) * N * B + na), ST::pack(fa[i]));
             if (hasb) {
 #pragma unroll
-                for (int i = 0; i < Q; ++i)
-                    __stcs(fout + (uint32_t(i) * N + nb), ST::pack(fb[i]));
+                for (int i = 0; i < Q; ++i) __stcs(at<kAddr>(fout, uint32_t(i) * N * B + nb), ST::pack(fb[i]));
             }
         } else {
             const int64_t na = (int64_t)blockIdx.x * kStepBlock + pair_node(threadIdx.x);
@@ -211,27 +217,18 @@ __global__ void ELBM_STEP_BOUNDS k_step(const typename ST::S *__restrict__ fin,
         const uint32_t sx[3] = {x == nx - 1 ? 0 : x + 1, x, x == 0 ? nx - 1 : x - 1};
         const uint32_t sy[3] = {y == ny - 1 ? 0 : (y + 1) * nx, y * nx, (y == 0 ? ny - 1 : y - 1) * nx};
         const uint32_t sz[3] = {z == nz - 1 ? 0 : z + 1, z, z == 0 ? nz - 1 : z - 1};
-        auto at = [](auto *base, uint32_t o) {
-            using P = decltype(base);
-            if constexpr (kAddr == kAddrBytes) {
-                using C = std::conditional_t<std::is_const_v<std::remove_pointer_t<P>>, const char, char>;
-                return reinterpret_cast<P>(reinterpret_cast<C *>(base) + o);
-            } else {
-                return base + o;
-            }
-        };
 #pragma unroll
         for (int i = 0; i < Q; ++i) {
             const int cx = vel(D, i, 0), cy = vel(D, i, 1), cz = D == 3 ? vel(D, i, 2) : 0;
             const uint32_t o = (sy[cy + 1] + sx[cx + 1]) * B;
             const uint32_t b = (uint32_t(i) * N + sz[cz + 1] * plane) * B;
-            f[i] = ST::raw(ld_pop<D == 3>(at(fin, o + b)));
+            f[i] = ST::raw(ld_pop<D == 3>(at<kAddr>(fin, o + b)));
         }
         collide_stored<D, ST, true>(f, xd, p, &br);
         if constexpr (kForce) add_force<D, T, ST::kDev>(f, p);
         const uint32_t n = (z * plane + xy) * B;
 #pragma unroll
-        for (int i = 0; i < Q; ++i) __stcs(at(fout, uint32_t(i) * N * B + n), ST::pack(f[i]));
+        for (int i = 0; i < Q; ++i) __stcs(at<kAddr>(fout, uint32_t(i) * N * B + n), ST::pack(f[i]));
     } else {
         const int64_t n = (int64_t)blockIdx.x * kStepBlock + threadIdx.x;
         if (n >= g.N) return;
@@ -1284,9 +1281,7 @@ cudaError_t ELBM_CAT(launch_step, ELBM_SUFFIX)(int storage, const void *fin, voi
                                           static_cast<const typename ST::S *>(fin),                    \
                                           static_cast<typename ST::S *>(fout), g, p, rd)));            \
     } else {                                                                                           \
-        ELBM_STORAGE_SWITCH(storage, (k_step<ST, (nodes_per_thread<D, ST>() == 2 && ADDR == kAddrBytes \
-                                                      ? kAddrElems                                     \
-                                                      : ADDR)><<<GRID, step_threads<ST>(), 0, s>>>(    \
+        ELBM_STORAGE_SWITCH(storage, (k_step<ST, ADDR><<<GRID, step_threads<ST>(), 0, s>>>(            \
                                           static_cast<const typename ST::S *>(fin),                    \
                                           static_cast<typename ST::S *>(fout), g, p, rd)));            \
     }
