@@ -1191,18 +1191,41 @@ __device__ __forceinline__ void collide2_stored(typename ST::T (&fa)[Lattice<D>:
     collide_stored<D, ST, kRelax>(fb, x, p, &br);
 }
 
+// ---------------------------------------------------------------------------
+// Kernels of one stream are launched with programmatic stream serialisation
+// (elbm_kernels.cuh: launch): the blocks of the next kernel may become resident while the
+// previous kernel drains, and wait here until it has completed and its writes are visible.
+// Every kernel calls this before it touches global memory.  Plain launches of dependent
+// kernels are at least 4.1 us apart on GB300 however small they are (measured on D2Q9 steps
+// of 1 to 128^2 nodes); this way a step of 64^2 takes 1.7 us, of 512^2 3.45 (6.16) and of
+// 1024^2 9.5 (12.3).  Triggering the next launch earlier (launch_dependents) was slower:
+// the waiting blocks take the room of the running ones.
+// Since such a kernel's life overlaps the previous kernel's writes, global data is read with
+// coherent loads (ld.global with a cache policy), never through the read-only path.
+// ---------------------------------------------------------------------------
+__device__ __forceinline__ void wait_previous_kernel() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 // Population loads of the step kernels.  D3Q27 loads with the evict-first (streaming)
 // policy (ld.global.cs): each line comes once from DRAM and is read again, within a few
 // warps, by the neighbours' shifted loads, while the register spills of the collision pass
 // through the same L1; population lines that leave first keep room for them (256^3 FP32
-// Taylor-Green start: 0.543 against 0.552 ms per step through the read-only path; 203 x 150
-// x 131 developed flow: 0.1525 against 0.157).  D2Q9, which does not spill to speak of, loads
-// through the read-only path.
+// Taylor-Green start: 0.543 against 0.552 ms per step without the policy; 203 x 150 x 131
+// developed flow: 0.1525 against 0.157).  D2Q9, which does not spill to speak of, loads
+// with the default policy.
 template <bool kStream, class S>
 __device__ __forceinline__ S ld_pop(const S *p)
 {
-    if constexpr (kStream) return __ldcs(p);
-    else return __ldg(p);
+    if constexpr (sizeof(S) == 2) { // the 16-bit intrinsics are not ordered behind wait_previous_kernel
+        const unsigned short *q = reinterpret_cast<const unsigned short *>(p);
+        unsigned short b;
+        if constexpr (kStream) b = __ldcs(q);
+        else b = __ldca(q);
+        return reinterpret_cast<S &>(b);
+    } else if constexpr (kStream) {
+        return __ldcs(p);
+    } else {
+        return __ldca(p);
+    }
 }
 
 // ---------------------------------------------------------------------------
@@ -1228,7 +1251,7 @@ __device__ __forceinline__ void pull_load(const typename ST::S *__restrict__ fin
         const int sy = cy == 1 ? ym : (cy == -1 ? yp : y);
         const int sz = cz == 1 ? zm : (cz == -1 ? zp : z);
         const int64_t src = ((int64_t)sz * g.ny + sy) * g.nx + sx;
-        const typename ST::S sv = __ldg(fin + (int64_t)i * g.N + src);
+        const typename ST::S sv = ld_pop<false>(fin + (int64_t)i * g.N + src);
         f[i] = kStep ? ST::raw(sv) : ST::load(sv, dev_ref<D, T>(i, R));
     }
 }

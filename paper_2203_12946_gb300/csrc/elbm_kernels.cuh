@@ -144,6 +144,7 @@ __global__ void ELBM_STEP_BOUNDS k_step(const typename ST::S *__restrict__ fin,
                                                     typename ST::S *__restrict__ fout, Geometry g,
                                                     CollideParams p, RowDiv rd)
 {
+    wait_previous_kernel();
     using S = typename ST::S;
     using T = typename ST::T;
     if constexpr (nodes_per_thread<D, ST>() == 2) {
@@ -359,21 +360,22 @@ __global__ void __launch_bounds__(kAuxBlock) k_init(const double *__restrict__ r
                                                    typename ST::S *__restrict__ f, Geometry g,
                                                    double rho_uniform, double rho0, int64_t n0, int64_t count)
 {
+    wait_previous_kernel();
     const int64_t k = (int64_t)blockIdx.x * kAuxBlock + threadIdx.x;
     if (k >= count) return;
     const int64_t n = n0 + k;
     double un[3] = {0.0, 0.0, 0.0}, feq[Q];
 #pragma unroll
-    for (int a = 0; a < D; ++a) un[a] = u[(int64_t)a * g.N + n];
+    for (int a = 0; a < D; ++a) un[a] = __ldcs(u + (int64_t)a * g.N + n);
     if constexpr (!ST::kDev && sizeof(typename ST::S) == 4) {
         // FP32 populations: the equilibrium in double-float, rounded once
         float fe[Q];
-        equilibrium_df(rho ? rho[n] : rho_uniform, un, fe);
+        equilibrium_df(rho ? __ldcs(rho + n) : rho_uniform, un, fe);
 #pragma unroll
         for (int i = 0; i < Q; ++i) f[(int64_t)i * g.N + n] = fe[i];
         return;
     }
-    equilibrium64<sizeof(typename ST::S) < 8>(rho ? rho[n] : rho_uniform, un, feq);
+    equilibrium64<sizeof(typename ST::S) < 8>(rho ? __ldcs(rho + n) : rho_uniform, un, feq);
     const double R = double(dev_unit<D>(rho0));
 #pragma unroll
     for (int i = 0; i < Q; ++i) f[(int64_t)i * g.N + n] = ST::store64(feq[i], weight_k(D, i) * R);
@@ -412,11 +414,12 @@ __device__ __forceinline__ double fixed_to_f64(long long q, int E0)
 // sums of the same values give whenever those are exact, without the FP64 pipe's rate; a
 // node holding a value that is not finite is summed in FP64.
 template <class ST>
-__global__ void __launch_bounds__(kAuxBlock) k_moments(const typename ST::S *__restrict__ f,
+__global__ void __launch_bounds__(kAuxBlock) k_moments(const typename ST::S *f,
                                                       Geometry g, double rho0,
-                                                      double *__restrict__ rho_out,
-                                                      double *__restrict__ u_out, int64_t n0, int64_t count)
+                                                      double *rho_out,
+                                                      double *u_out, int64_t n0, int64_t count)
 {
+    wait_previous_kernel();
     const int64_t k = (int64_t)blockIdx.x * kAuxBlock + threadIdx.x;
     if (k >= count) return;
     const int64_t n = n0 + k;
@@ -479,6 +482,7 @@ __global__ void __launch_bounds__(kStepBlock) k_alpha(const typename ST::S *__re
                                                      uint8_t *__restrict__ flags,
                                                      double *__restrict__ nut_out)
 {
+    wait_previous_kernel();
     using T = typename ST::T;
     const int64_t n = (int64_t)blockIdx.x * kStepBlock + threadIdx.x;
     if (n >= g.N) return;
@@ -715,6 +719,7 @@ __global__ void __launch_bounds__(kAuxBlock) k_diag(const typename ST::S *__rest
                                                    Geometry g, CollideParams p,
                                                    DiagAcc *__restrict__ acc)
 {
+    wait_previous_kernel();
     using T = typename ST::T;
     __shared__ unsigned int s_hist[ELBM_HIST_BINS + 2];
     for (int b = threadIdx.x; b < ELBM_HIST_BINS + 2; b += kAuxBlock) s_hist[b] = 0u;
@@ -751,6 +756,7 @@ __global__ void __launch_bounds__(kStepBlock, step_diag_min_blocks<ST>()) k_step
                                              typename ST::S *__restrict__ fout, Geometry g, CollideParams p,
                                              DiagAcc *__restrict__ acc)
 {
+    wait_previous_kernel();
     using T = typename ST::T;
     __shared__ unsigned int s_hist[ELBM_HIST_BINS + 2];
     for (int b = threadIdx.x; b < ELBM_HIST_BINS + 2; b += kStepBlock) s_hist[b] = 0u;
@@ -868,6 +874,7 @@ __global__ void __launch_bounds__(BX / nodes_per_thread<D, ST>(), batch_min_bloc
                                                   typename ST::S *__restrict__ fout,
                                                   const __grid_constant__ BatchTable tab, CollideParams p)
 {
+    wait_previous_kernel();
     using T = typename ST::T;
     const int bid = int(blockIdx.x);
     int lo = tab.coarse[bid >> tab.shift]; // item0[lo] <= bid
@@ -1033,6 +1040,7 @@ __global__ void __launch_bounds__(kAuxBlock) k_step_adjoint(const typename ST::S
                                                            typename ST::T *__restrict__ gout, Geometry g,
                                                            CollideParams p, double *__restrict__ dforce)
 {
+    wait_previous_kernel();
     using T = typename ST::T;
     const int64_t n = (int64_t)blockIdx.x * kAuxBlock + threadIdx.x;
     T dfl[3] = {T(0), T(0), T(0)};
@@ -1042,7 +1050,7 @@ __global__ void __launch_bounds__(kAuxBlock) k_step_adjoint(const typename ST::S
         T F[Q], gl[Q], h[Q];
         pull_load<D, ST>(fin, g, x, y, z, p.dunit_f, F);
 #pragma unroll
-        for (int i = 0; i < Q; ++i) gl[i] = gnext[(int64_t)i * g.N + n];
+        for (int i = 0; i < Q; ++i) gl[i] = __ldcs(gnext + (int64_t)i * g.N + n);
         node_vjp<D, T, kForce>(F, gl, p, h, dfl);
         const int xm = x == 0 ? g.nx - 1 : x - 1, xp = x == g.nx - 1 ? 0 : x + 1;
         const int ym = y == 0 ? g.ny - 1 : y - 1, yp = y == g.ny - 1 ? 0 : y + 1;
@@ -1081,6 +1089,7 @@ __global__ void __launch_bounds__(kAuxBlock) k_kinetic_energy(const typename ST:
                                                              Geometry g, double rho0, double *__restrict__ acc,
                                                              typename ST::T *__restrict__ grad)
 {
+    wait_previous_kernel();
     using T = typename ST::T;
     double e = 0.0;
     const double R = double(dev_unit<D>(rho0));
@@ -1089,7 +1098,7 @@ __global__ void __launch_bounds__(kAuxBlock) k_kinetic_energy(const typename ST:
         double fv[Q];
 #pragma unroll
         for (int i = 0; i < Q; ++i) {
-            fv[i] = ST::load64(f[(int64_t)i * g.N + n], weight_k(D, i) * R);
+            fv[i] = ST::load64(ld_pop<true>(f + (int64_t)i * g.N + n), weight_k(D, i) * R);
             r += fv[i];
 #pragma unroll
             for (int a = 0; a < D; ++a) j[a] += vel(D, i, a) * fv[i];
@@ -1123,13 +1132,14 @@ __global__ void __launch_bounds__(kAuxBlock) k_equilibrium_vjp(const double *__r
                                                               const T *__restrict__ gf, Geometry g, double rho_uniform,
                                                               double *__restrict__ drho, double *__restrict__ du)
 {
+    wait_previous_kernel();
     const int64_t n = (int64_t)blockIdx.x * kAuxBlock + threadIdx.x;
     if (n >= g.N) return;
-    const double r = rho ? rho[n] : rho_uniform;
+    const double r = rho ? __ldcs(rho + n) : rho_uniform;
     double phi[3][3], dlp[3][3];
 #pragma unroll
     for (int a = 0; a < D; ++a) {
-        const double ua = u[(int64_t)a * g.N + n];
+        const double ua = __ldcs(u + (int64_t)a * g.N + n);
         const double s = sqrt(1.0 + 3.0 * ua * ua), Y = 2.0 - s, num = 2.0 * ua + s, den = 1.0 - ua;
         const double zz = num / den, dY = -3.0 * ua / s, dlz = (2.0 + 3.0 * ua / s) / num + 1.0 / den;
         phi[a][0] = Y / (6.0 * zz);
@@ -1145,7 +1155,7 @@ __global__ void __launch_bounds__(kAuxBlock) k_equilibrium_vjp(const double *__r
         double v = r;
 #pragma unroll
         for (int a = 0; a < D; ++a) v *= phi[a][vel(D, i, a) + 1];
-        const double gv = double(gf[(int64_t)i * g.N + n]) * v;
+        const double gv = double(__ldcs(gf + (int64_t)i * g.N + n)) * v;
         sr += gv;
 #pragma unroll
         for (int a = 0; a < D; ++a) su[a] += gv * dlp[a][vel(D, i, a) + 1];
@@ -1171,6 +1181,24 @@ __global__ void __launch_bounds__(kAuxBlock) k_equilibrium_vjp(const double *__r
     }
 
 static inline unsigned blocks_for(int64_t N, int block) { return unsigned((N + block - 1) / block); }
+
+// Launches a kernel that begins with wait_previous_kernel().
+template <class... P, class... A>
+cudaError_t launch(void (*kernel)(P...), dim3 grid, unsigned block, cudaStream_t s, A &&...args)
+{
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(block);
+    cfg.stream = s;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+    if (e != cudaSuccess) cudaGetLastError(); // reported here, not by the caller's next CUDA call
+    return e;
+}
 
 } // namespace ELBM_SUFFIX
 
@@ -1276,14 +1304,14 @@ cudaError_t ELBM_CAT(launch_step, ELBM_SUFFIX)(int storage, const void *fin, voi
     const RowDiv rd = row_div(uint32_t(g.nx));
 #define ELBM_DIRECT_STEP(ADDR, GRID)                                                                   \
     if (forced) {                                                                                      \
-        ELBM_STORAGE_SWITCH(storage, (k_step<ST, (ADDR == kAddrBytes ? kAddrElems : ADDR), true>       \
-                                      <<<GRID, step_threads<ST>(), 0, s>>>(                            \
-                                          static_cast<const typename ST::S *>(fin),                    \
-                                          static_cast<typename ST::S *>(fout), g, p, rd)));            \
+        ELBM_STORAGE_SWITCH(storage, return launch(k_step<ST, (ADDR == kAddrBytes ? kAddrElems : ADDR), true>, \
+                                                   GRID, step_threads<ST>(), s,                        \
+                                                   static_cast<const typename ST::S *>(fin),           \
+                                                   static_cast<typename ST::S *>(fout), g, p, rd))     \
     } else {                                                                                           \
-        ELBM_STORAGE_SWITCH(storage, (k_step<ST, ADDR><<<GRID, step_threads<ST>(), 0, s>>>(            \
-                                          static_cast<const typename ST::S *>(fin),                    \
-                                          static_cast<typename ST::S *>(fout), g, p, rd)));            \
+        ELBM_STORAGE_SWITCH(storage, return launch(k_step<ST, ADDR>, GRID, step_threads<ST>(), s,      \
+                                                   static_cast<const typename ST::S *>(fin),           \
+                                                   static_cast<typename ST::S *>(fout), g, p, rd))     \
     }
     const bool pair = D == 2 && storage != ELBM_STORE_F64; // two nodes per thread, blocks along rows
     const int64_t plane = int64_t(g.nx) * g.ny;
@@ -1319,9 +1347,9 @@ cudaError_t ELBM_CAT(launch_step_diag, ELBM_SUFFIX)(int storage, const void *fin
     const uint64_t items = uint64_t((g.nx + kStepBlock - 1) / kStepBlock) * uint64_t(g.ny) * uint64_t(g.nz);
     const uint64_t cap = uint64_t(num_sms > 0 ? num_sms : 1) * 8u;
     const unsigned grid = unsigned(items < cap ? items : cap);
-    ELBM_STORAGE_SWITCH(storage, (k_step_diag<ST><<<grid, kStepBlock, 0, s>>>(
-                                     static_cast<const typename ST::S *>(fin), static_cast<typename ST::S *>(fout),
-                                     g, p, acc)));
+    ELBM_STORAGE_SWITCH(storage, return launch(k_step_diag<ST>, grid, kStepBlock, s,
+                                               static_cast<const typename ST::S *>(fin),
+                                               static_cast<typename ST::S *>(fout), g, p, acc))
     return cudaGetLastError();
 }
 
@@ -1333,9 +1361,9 @@ cudaError_t ELBM_CAT(launch_step_batch, ELBM_SUFFIX)(int storage, const void *fi
     const int nitems = tab.item0[tab.n];
     if (tab.n <= 0 || nitems <= 0) return cudaSuccess;
 #define ELBM_BATCH_BX(BXV)                                                                             \
-    ELBM_STORAGE_SWITCH(storage, (k_step_batch<ST, BXV><<<unsigned(nitems), BXV / nodes_per_thread<D, ST>(), 0, s>>>( \
-                                     static_cast<const typename ST::S *>(fin),                          \
-                                     static_cast<typename ST::S *>(fout), tab, p)))
+    ELBM_STORAGE_SWITCH(storage, return launch(k_step_batch<ST, BXV>, unsigned(nitems), BXV / nodes_per_thread<D, ST>(), s, \
+                                               static_cast<const typename ST::S *>(fin),               \
+                                               static_cast<typename ST::S *>(fout), tab, p))
     switch (bx) {
     case 64: ELBM_BATCH_BX(64); break;
     case 128: ELBM_BATCH_BX(128); break;
@@ -1402,15 +1430,15 @@ cudaError_t ELBM_CAT(launch_step_adjoint, ELBM_SUFFIX)(int storage, const void *
     if (g.N == 0) return cudaSuccess;
     const bool forced = dforce || p.force[0] != 0.0 || p.force[1] != 0.0 || p.force[2] != 0.0;
     if (forced) {
-        ELBM_STORAGE_SWITCH(storage, (k_step_adjoint<ST, true><<<blocks_for(g.N, kAuxBlock), kAuxBlock, 0, s>>>(
-                                         static_cast<const typename ST::S *>(fin),
-                                         static_cast<const typename ST::T *>(gnext),
-                                         static_cast<typename ST::T *>(gout), g, p, dforce)));
+        ELBM_STORAGE_SWITCH(storage, return launch(k_step_adjoint<ST, true>, blocks_for(g.N, kAuxBlock),
+                                                   kAuxBlock, s, static_cast<const typename ST::S *>(fin),
+                                                   static_cast<const typename ST::T *>(gnext),
+                                                   static_cast<typename ST::T *>(gout), g, p, dforce))
     } else {
-        ELBM_STORAGE_SWITCH(storage, (k_step_adjoint<ST><<<blocks_for(g.N, kAuxBlock), kAuxBlock, 0, s>>>(
-                                         static_cast<const typename ST::S *>(fin),
-                                         static_cast<const typename ST::T *>(gnext),
-                                         static_cast<typename ST::T *>(gout), g, p, nullptr)));
+        ELBM_STORAGE_SWITCH(storage, return launch(k_step_adjoint<ST>, blocks_for(g.N, kAuxBlock), kAuxBlock,
+                                                   s, static_cast<const typename ST::S *>(fin),
+                                                   static_cast<const typename ST::T *>(gnext),
+                                                   static_cast<typename ST::T *>(gout), g, p, nullptr))
     }
     return cudaGetLastError();
 }
@@ -1423,9 +1451,9 @@ cudaError_t ELBM_CAT(launch_kinetic_energy, ELBM_SUFFIX)(int storage, const void
     unsigned blocks = blocks_for(g.N, kAuxBlock);
     const unsigned cap = unsigned(num_sms > 0 ? num_sms : 1) * 8u;
     if (blocks > cap) blocks = cap;
-    ELBM_STORAGE_SWITCH(storage, (k_kinetic_energy<ST><<<blocks, kAuxBlock, 0, s>>>(
-                                     static_cast<const typename ST::S *>(f), g, rho0, acc,
-                                     static_cast<typename ST::T *>(grad))));
+    ELBM_STORAGE_SWITCH(storage, return launch(k_kinetic_energy<ST>, blocks, kAuxBlock, s,
+                                               static_cast<const typename ST::S *>(f), g, rho0, acc,
+                                               static_cast<typename ST::T *>(grad)))
     return cudaGetLastError();
 }
 
@@ -1436,12 +1464,10 @@ cudaError_t ELBM_CAT(launch_equilibrium_vjp, ELBM_SUFFIX)(int storage, const dou
     using namespace ELBM_SUFFIX;
     if (g.N == 0) return cudaSuccess;
     if (storage == ELBM_STORE_F64)
-        k_equilibrium_vjp<double><<<blocks_for(g.N, kAuxBlock), kAuxBlock, 0, s>>>(
-            rho, u, static_cast<const double *>(gf), g, rho_uniform, drho, du);
-    else
-        k_equilibrium_vjp<float><<<blocks_for(g.N, kAuxBlock), kAuxBlock, 0, s>>>(
-            rho, u, static_cast<const float *>(gf), g, rho_uniform, drho, du);
-    return cudaGetLastError();
+        return launch(k_equilibrium_vjp<double>, blocks_for(g.N, kAuxBlock), kAuxBlock, s, rho, u, static_cast<const double *>(gf), g,
+                      rho_uniform, drho, du);
+    return launch(k_equilibrium_vjp<float>, blocks_for(g.N, kAuxBlock), kAuxBlock, s, rho, u, static_cast<const float *>(gf), g,
+                  rho_uniform, drho, du);
 }
 
 cudaError_t ELBM_CAT(launch_init, ELBM_SUFFIX)(int storage, const double *rho, const double *u,
@@ -1450,8 +1476,9 @@ cudaError_t ELBM_CAT(launch_init, ELBM_SUFFIX)(int storage, const double *rho, c
 {
     using namespace ELBM_SUFFIX;
     if (count <= 0) return cudaSuccess;
-    ELBM_STORAGE_SWITCH(storage, (k_init<ST><<<blocks_for(count, kAuxBlock), kAuxBlock, 0, s>>>(
-                                     rho, u, static_cast<typename ST::S *>(f), g, rho_uniform, rho0, n0, count)));
+    ELBM_STORAGE_SWITCH(storage, return launch(k_init<ST>, blocks_for(count, kAuxBlock), kAuxBlock, s, rho,
+                                               u, static_cast<typename ST::S *>(f), g, rho_uniform, rho0, n0,
+                                               count))
     return cudaGetLastError();
 }
 
@@ -1461,8 +1488,9 @@ cudaError_t ELBM_CAT(launch_moments, ELBM_SUFFIX)(int storage, const void *f, co
 {
     using namespace ELBM_SUFFIX;
     if (count <= 0) return cudaSuccess;
-    ELBM_STORAGE_SWITCH(storage, (k_moments<ST><<<blocks_for(count, kAuxBlock), kAuxBlock, 0, s>>>(
-                                     static_cast<const typename ST::S *>(f), g, rho0, rho_out, u_out, n0, count)));
+    ELBM_STORAGE_SWITCH(storage, return launch(k_moments<ST>, blocks_for(count, kAuxBlock), kAuxBlock, s,
+                                               static_cast<const typename ST::S *>(f), g, rho0, rho_out,
+                                               u_out, n0, count))
     return cudaGetLastError();
 }
 
@@ -1472,8 +1500,9 @@ cudaError_t ELBM_CAT(launch_alpha, ELBM_SUFFIX)(int storage, const void *f, cons
 {
     using namespace ELBM_SUFFIX;
     if (g.N == 0) return cudaSuccess;
-    ELBM_STORAGE_SWITCH(storage, (k_alpha<ST><<<blocks_for(g.N, kStepBlock), kStepBlock, 0, s>>>(
-                                     static_cast<const typename ST::S *>(f), g, p, alpha_out, flags, nut_out)));
+    ELBM_STORAGE_SWITCH(storage, return launch(k_alpha<ST>, blocks_for(g.N, kStepBlock), kStepBlock, s,
+                                               static_cast<const typename ST::S *>(f), g, p, alpha_out,
+                                               flags, nut_out))
     return cudaGetLastError();
 }
 
@@ -1486,8 +1515,8 @@ cudaError_t ELBM_CAT(launch_diag, ELBM_SUFFIX)(int storage, const void *f, const
     unsigned blocks = blocks_for(g.N, kAuxBlock);
     const unsigned cap = unsigned(num_sms > 0 ? num_sms : 1) * 8u;
     if (blocks > cap) blocks = cap;
-    ELBM_STORAGE_SWITCH(storage, (k_diag<ST><<<blocks, kAuxBlock, 0, s>>>(
-                                     static_cast<const typename ST::S *>(f), g, p, acc)));
+    ELBM_STORAGE_SWITCH(storage, return launch(k_diag<ST>, blocks, kAuxBlock, s,
+                                               static_cast<const typename ST::S *>(f), g, p, acc))
     return cudaGetLastError();
 }
 
