@@ -209,7 +209,7 @@ __global__ void ELBM_STEP_BOUNDS k_step(const typename ST::S *__restrict__ fin,
     int br;
     if constexpr (kAddr != kAddrWide) {
         const uint32_t nx = uint32_t(g.nx), ny = uint32_t(g.ny), nz = uint32_t(g.nz), N = uint32_t(g.N);
-        const uint32_t plane = nx * ny, xy = blockIdx.x * kStepBlock + threadIdx.x, z = blockIdx.y;
+        const uint32_t plane = nx * ny, xy = blockIdx.x * blockDim.x + threadIdx.x, z = blockIdx.y;
         if (xy >= plane) return;
         const uint32_t y = div_row(xy, rd), x = xy - y * nx;
         // offsets of the nine (c_x, c_y) sources in a plane; the rest of an address is the
@@ -1305,21 +1305,28 @@ cudaError_t ELBM_CAT(launch_step, ELBM_SUFFIX)(int storage, const void *fin, voi
 #define ELBM_DIRECT_STEP(ADDR, GRID)                                                                   \
     if (forced) {                                                                                      \
         ELBM_STORAGE_SWITCH(storage, return launch(k_step<ST, (ADDR == kAddrBytes ? kAddrElems : ADDR), true>, \
-                                                   GRID, step_threads<ST>(), s,                        \
+                                                   GRID, threads, s,                                   \
                                                    static_cast<const typename ST::S *>(fin),           \
                                                    static_cast<typename ST::S *>(fout), g, p, rd))     \
     } else {                                                                                           \
-        ELBM_STORAGE_SWITCH(storage, return launch(k_step<ST, ADDR>, GRID, step_threads<ST>(), s,      \
+        ELBM_STORAGE_SWITCH(storage, return launch(k_step<ST, ADDR>, GRID, threads, s,                 \
                                                    static_cast<const typename ST::S *>(fin),           \
                                                    static_cast<typename ST::S *>(fout), g, p, rd))     \
     }
     const bool pair = D == 2 && storage != ELBM_STORE_F64; // two nodes per thread, blocks along rows
     const int64_t plane = int64_t(g.nx) * g.ny;
     if (elems > 0xffffffffull || (pair ? g.ny : g.nz) > 65535) {
+        const unsigned threads = pair ? step_threads<StoreF32>() : kStepBlock;
         ELBM_DIRECT_STEP(kAddrWide, blocks_for(g.N, kStepBlock))
     } else {
+        // one node per thread: smaller blocks where full ones would leave SMs without work (D2Q9
+        // FP64, 96^2: 55 us per step in blocks of 256, 28 so); FP64 is bound by each SM's FP64
+        // pipe and takes 64 from the start, which divides the nodes more evenly over the SMs
+        unsigned threads = pair ? step_threads<StoreF32>() : storage == ELBM_STORE_F64 ? 64u : unsigned(kStepBlock);
+        if (!pair)
+            while (threads > 32 && int64_t(blocks_for(plane, threads)) * g.nz < 2 * int64_t(num_sms)) threads /= 2;
         const dim3 grid = pair ? dim3(blocks_for(g.nx, kStepBlock), unsigned(g.ny))
-                               : dim3(blocks_for(plane, kStepBlock), unsigned(g.nz));
+                               : dim3(blocks_for(plane, threads), unsigned(g.nz));
         const uint64_t size = storage == ELBM_STORE_F64                                       ? 8
                               : storage == ELBM_STORE_F32 || storage == ELBM_STORE_F32DEV ? 4
                                                                                               : 2;
