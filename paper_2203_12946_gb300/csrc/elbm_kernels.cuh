@@ -243,29 +243,31 @@ __global__ void ELBM_STEP_BOUNDS k_step(const typename ST::S *__restrict__ fin,
     }
 }
 
-// FP64 equilibrium from rho and u (same product form as node_collide).  Per axis
-// phi(-1) = Y den / (6 num) and phi(+1) = Y num / (6 den); with kOneDiv they share one
-// division, r = Y / (6 num den), phi(-1) = r den^2, phi(+1) = r num^2 (a few FP64 ulp
-// apart: used where the result is rounded to FP32 or below).
-template <bool kOneDiv>
+// FP64 equilibrium from rho and u (same product form as node_collide): per axis
+// phi(-1) = Y den / (6 num) and phi(+1) = Y num / (6 den); kDivide = false takes the same
+// factors as (1 + 2t -+ 3u) / 6 with t = s - 1 (to about 2^-51 f^eq), for the nodes that
+// k_init evaluates again before rounding them to FP32.
+template <bool kDivide>
 __device__ __forceinline__ void equilibrium64(double rho, const double (&u)[3], double (&feq)[Q])
 {
     double phi[3][3];
 #pragma unroll
     for (int a = 0; a < D; ++a) {
         const double s = sqrt(1.0 + 3.0 * u[a] * u[a]);
-        const double Y = 2.0 - s;
-        const double num = 2.0 * u[a] + s, den = 1.0 - u[a];
-        if (kOneDiv) {
-            const double r = Y / (6.0 * num * den);
-            phi[a][0] = r * den * den;
-            phi[a][2] = r * num * num;
-        } else {
+        if constexpr (kDivide) {
+            const double Y = 2.0 - s;
+            const double num = 2.0 * u[a] + s, den = 1.0 - u[a];
             phi[a][0] = Y * den / (6.0 * num);
+            phi[a][1] = Y * (4.0 / 6.0);
             phi[a][2] = Y * num / (6.0 * den);
+        } else {
+            const double q = fma(2.0, s, -1.0);
+            phi[a][0] = fma(-3.0, u[a], q);
+            phi[a][1] = fma(-4.0, s, 8.0);
+            phi[a][2] = fma(3.0, u[a], q);
         }
-        phi[a][1] = Y * (4.0 / 6.0);
     }
+    if constexpr (!kDivide) rho *= weight_unit(D);
 #pragma unroll
     for (int i = 0; i < Q; ++i) {
         double v = rho;
@@ -287,10 +289,28 @@ __device__ __forceinline__ DF df_fast_two_sum(float a, float b) // |a| >= |b|
     const float s = a + b;
     return {s, b - (s - a)};
 }
+// An FP64 value as hi, the nearest FP32 number, and lo, the rest rounded to FP32, on the
+// integer pipe: a conversion or an FP64 addition occupies GB300's FP64 pipe for 16 cycles per
+// warp and SM, and four values converted through it (16 such instructions) bounded the whole
+// kernel.  Below 2^-74 lo, and below 2^-126 the value, is flushed to zero; values beyond
+// FP32's range, infinities and NaN give infinities and NaN.
 __device__ __forceinline__ DF df_from_double(double x)
 {
-    const float h = __double2float_rn(x);
-    return {h, __double2float_rn(x - double(h))};
+    const uint64_t b = (uint64_t)__double_as_longlong(x);
+    const uint32_t top = uint32_t(b >> 32), sign = top & 0x80000000u;
+    const int e = int((top >> 20) & 0x7ffu) - 896; // FP32's biased exponent
+    if (e <= 0) return {__uint_as_float(sign), 0.0f};
+    if (e >= 255) { // NaN stays NaN, anything else is infinite
+        const bool nan = (top & 0x7fffffffu) > 0x7ff00000u || ((top & 0x7fffffffu) == 0x7ff00000u && uint32_t(b) != 0);
+        return {__uint_as_float(sign | (nan ? 0x7fc00000u : 0x7f800000u)), 0.0f};
+    }
+    // the 23 leading bits of the significand, rounded to nearest even by the other 29 (a carry
+    // runs into the exponent, as it should)
+    const uint32_t m = (uint32_t(e) << 23) | (uint32_t(b >> 29) & 0x7fffffu), low = uint32_t(b) & 0x1fffffffu;
+    const uint32_t up = low > 0x10000000u || (low == 0x10000000u && (m & 1u)) ? 1u : 0u;
+    const float rest = float(int(low) - int(up << 29)); // in units of 2^(e - 127 - 52)
+    const float scale = e > 52 ? __uint_as_float(sign | (uint32_t(e - 52) << 23)) : 0.0f;
+    return {__uint_as_float(sign | (m + up)), rest * scale};
 }
 __device__ __forceinline__ DF df_add(DF a, DF b)
 {
@@ -311,6 +331,7 @@ __device__ __forceinline__ DF df_mulf(DF a, float b)
     const float p = a.hi * b;
     return df_fast_two_sum(p, fmaf(a.lo, b, fmaf(a.hi, b, -p)));
 }
+__device__ __forceinline__ DF df_neg(DF a) { return {-a.hi, -a.lo}; }
 __device__ __forceinline__ DF df_div(DF a, DF b)
 {
     const float q = a.hi / b.hi;
@@ -325,35 +346,78 @@ __device__ __forceinline__ DF df_sqrt(DF a)
     return df_fast_two_sum(r, e / (2.0f * r));
 }
 
-// The equilibrium of equilibrium64<true> in double-float: f^eq rounded once to FP32
-// (|stored - f^eq| <= half an FP32 ulp + 2^-43 f^eq), without the FP64 pipe.
-__device__ __forceinline__ void equilibrium_df(double rho, const double (&u)[3], float (&feq)[Q])
+// The equilibrium in double-float, less k_i R (R = 0: populations), rounded once to FP32:
+// |error| <= half an FP32 ulp + about 2^-44 f^eq.  Per axis phi(-1) = Y den / (6 num) and
+// phi(+1) = Y num / (6 den) share one division, r = Y / (6 num den), phi(-1) = r den^2,
+// phi(+1) = r num^2.  Returns whether every value is known to be the correctly rounded one
+// (only with kSure: f^eq - k_i R is small, so 2^-44 f^eq can reach its last bit): the error
+// term of the sum is further than 2^-44 f^eq from half an ulp of the result.
+template <bool kSure>
+__device__ __forceinline__ bool equilibrium_df(DF rho, const DF (&u)[3], float R, float (&feq)[Q])
 {
     constexpr double kTwoThirds = 2.0 / 3.0;
     const DF two3 = {float(kTwoThirds), float(kTwoThirds - double(float(kTwoThirds)))};
     DF phi[3][3];
 #pragma unroll
     for (int a = 0; a < D; ++a) {
-        const DF U = df_from_double(u[a]);
+        const DF U = u[a];
         const DF S = df_sqrt(df_add({1.0f, 0.0f}, df_mulf(df_mul(U, U), 3.0f)));
-        const DF Y = df_add({2.0f, 0.0f}, {-S.hi, -S.lo});
-        const DF num = df_add({2.0f * U.hi, 2.0f * U.lo}, S), den = df_add({1.0f, 0.0f}, {-U.hi, -U.lo});
+        const DF Y = df_add({2.0f, 0.0f}, df_neg(S));
+        const DF num = df_add({2.0f * U.hi, 2.0f * U.lo}, S), den = df_add({1.0f, 0.0f}, df_neg(U));
         const DF r = df_div(Y, df_mulf(df_mul(num, den), 6.0f));
         phi[a][0] = df_mul(r, df_mul(den, den));
         phi[a][1] = df_mul(Y, two3);
         phi[a][2] = df_mul(r, df_mul(num, num));
     }
-    const DF R = df_from_double(rho);
+    bool sure = true;
+    DF v[Q / 3]; // rho times the factors of all axes but the last
 #pragma unroll
-    for (int i = 0; i < Q; ++i) {
-        DF v = R;
+    for (int x = 0; x < 3; ++x) {
+        const DF rx = df_mul(rho, phi[0][x]);
+        if constexpr (D == 2) {
+            v[x] = rx;
+        } else {
 #pragma unroll
-        for (int a = 0; a < D; ++a) v = df_mul(v, phi[a][vel(D, i, a) + 1]);
-        feq[i] = v.hi;
+            for (int y = 0; y < 3; ++y) v[3 * x + y] = df_mul(rx, phi[1][y]);
+        }
     }
+    // the last axis: c = -1 and +1 on packed pairs; en = -(error of p)
+    const DF b0 = phi[D - 1][0], b1 = phi[D - 1][1], b2 = phi[D - 1][2];
+    const float2 bh = f2(b0.hi, b2.hi), bl = f2(b0.lo, b2.lo);
+    auto put = [&](int i, float p, float en) {
+        const float c = -float(weight_k(D, i)) * R, d = p + c;
+        if constexpr (kSure) {
+            const float dd = d - p;
+            const float w = ((p - (d - dd)) + (c - dd)) - en; // what p + c - d lost, and p's error
+            const float r1 = d + w, err = w - (r1 - d);
+            const float half_ulp = __uint_as_float(max(__float_as_uint(r1) & 0x7f800000u, 24u << 23) - (24u << 23));
+            sure = sure && fabsf(fabsf(err) - half_ulp) > 0x1p-44f * p;
+            feq[i] = r1;
+        } else {
+            feq[i] = d - en;
+        }
+    };
+#pragma unroll
+    for (int k = 0; k < Q / 3; ++k) {
+        const DF a = v[k];
+        const float2 p2 = pmul(f2(a.hi), bh);
+        const float2 e2 = pfma(f2(-a.lo), bh, pfma(f2(-a.hi), bl, pfma(f2(-a.hi), bh, p2)));
+        const float p1 = a.hi * b1.hi, e1 = fmaf(-a.lo, b1.hi, fmaf(-a.hi, b1.lo, fmaf(-a.hi, b1.hi, p1)));
+        put(3 * k, p2.x, e2.x);
+        put(3 * k + 1, p1, e1);
+        put(3 * k + 2, p2.y, e2.y);
+    }
+    return sure;
 }
 
-// f = f^eq(rho, u) for the nodes n0 .. n0 + count - 1 (SoA with stride g.N).
+// f = f^eq(rho, u) for the nodes n0 .. n0 + count - 1 (SoA with stride g.N).  FP64 storage
+// in FP64; the FP32-arithmetic storages in double-float (equilibrium_df), rounded once to
+// FP32 (then to 16 bits), but for a node whose FP32 deviations are not sure to be rounded as
+// FP64 would (a few nodes in a hundred): FP64 again.  4.8 M D3Q27 nodes: 145 us for FP32
+// populations (158 with FP64 conversions), 228 for FP32 deviations and 151 for FP16 (1 433 in
+// FP64); 8 M D2Q9 nodes: 133, 171 and 138 (184, 1 249, 1 250).  Bound by the FP32 arithmetic and
+// its issue slots.  The factors without divisions (1 + 2t -+ 3u) take 122 and 108 us, but round
+// a few values in 10^8 the other way than this form, which would show in FP64 moments.
 template <class ST>
 __global__ void __launch_bounds__(kAuxBlock) k_init(const double *__restrict__ rho,
                                                    const double *__restrict__ u,
@@ -364,18 +428,23 @@ __global__ void __launch_bounds__(kAuxBlock) k_init(const double *__restrict__ r
     const int64_t k = (int64_t)blockIdx.x * kAuxBlock + threadIdx.x;
     if (k >= count) return;
     const int64_t n = n0 + k;
-    double un[3] = {0.0, 0.0, 0.0}, feq[Q];
+    const double r = rho ? __ldcs(rho + n) : rho_uniform;
+    double un[3] = {0.0, 0.0, 0.0};
 #pragma unroll
     for (int a = 0; a < D; ++a) un[a] = __ldcs(u + (int64_t)a * g.N + n);
-    if constexpr (!ST::kDev && sizeof(typename ST::S) == 4) {
-        // FP32 populations: the equilibrium in double-float, rounded once
+    if constexpr (sizeof(typename ST::T) == 4) {
+        const DF ud[3] = {df_from_double(un[0]), df_from_double(un[1]), df_from_double(un[2])};
         float fe[Q];
-        equilibrium_df(rho ? __ldcs(rho + n) : rho_uniform, un, fe);
+        const float R = ST::kDev ? dev_unit<D>(rho0) : 0.0f;
+        const bool sure = equilibrium_df<ST::kDevCollide>(df_from_double(r), ud, R, fe);
+        if (!ST::kDevCollide || sure) {
 #pragma unroll
-        for (int i = 0; i < Q; ++i) f[(int64_t)i * g.N + n] = fe[i];
-        return;
+            for (int i = 0; i < Q; ++i) f[(int64_t)i * g.N + n] = ST::pack(fe[i]);
+            return;
+        }
     }
-    equilibrium64<sizeof(typename ST::S) < 8>(rho ? __ldcs(rho + n) : rho_uniform, un, feq);
+    double feq[Q];
+    equilibrium64<sizeof(typename ST::T) == 8>(r, un, feq);
     const double R = double(dev_unit<D>(rho0));
 #pragma unroll
     for (int i = 0; i < Q; ++i) f[(int64_t)i * g.N + n] = ST::store64(feq[i], weight_k(D, i) * R);
@@ -407,53 +476,141 @@ __device__ __forceinline__ double fixed_to_f64(long long q, int E0)
     return double(q) * __longlong_as_double((long long)(E0 - 150 + 1023) << 52);
 }
 
-// rho and u of the stored state (FP64) for the nodes n0 .. n0 + count - 1.  FP64 storage
-// sums in FP64.  The FP32-arithmetic storages hold FP32 values (populations, or deviations
-// d_i of the reference c_i = k_i R with sum_i c_i = 6^D R and sum_i c_i c_i = 0): their sums
-// are taken exactly in fixed point (f32_fixed) and rounded once to FP64, the result the FP64
-// sums of the same values give whenever those are exact, without the FP64 pipe's rate; a
-// node holding a value that is not finite is summed in FP64.
+// A finite FP32 value that is zero or normal as FP64, on the integer pipe.
+__device__ __forceinline__ double f32_to_f64(float v)
+{
+    const uint32_t b = __float_as_uint(v);
+    const uint32_t hi = (b & 0x80000000u) | (((b >> 3) & 0x0fffffffu) + (896u << 20));
+    return (b << 1) ? __hiloint2double(int(hi), int(b << 29)) : 0.0;
+}
+
+// Sums of a over the node (r) and of c_a a (j), any order (the values add exactly).
+__device__ __forceinline__ void lattice_sums(const float (&a)[Q], float &r, float (&j)[3])
+{
+    constexpr int P = Q / 3;
+    float s0[P], s1[P];
+#pragma unroll
+    for (int k = 0; k < P; ++k) s0[k] = a[3 * k] + a[3 * k + 1] + a[3 * k + 2], s1[k] = a[3 * k + 2] - a[3 * k];
+    if constexpr (D == 2) {
+        r = s0[0] + s0[1] + s0[2];
+        j[0] = s0[2] - s0[0];
+        j[1] = s1[0] + s1[1] + s1[2];
+    } else {
+        float t[3], ty[3], tz[3];
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            t[k] = s0[3 * k] + s0[3 * k + 1] + s0[3 * k + 2];
+            ty[k] = s0[3 * k + 2] - s0[3 * k];
+            tz[k] = s1[3 * k] + s1[3 * k + 1] + s1[3 * k + 2];
+        }
+        r = t[0] + t[1] + t[2];
+        j[0] = t[2] - t[0];
+        j[1] = ty[0] + ty[1] + ty[2];
+        j[2] = tz[0] + tz[1] + tz[2];
+    }
+}
+
+// rho and rho u of a node from its stored FP32 values (populations, or deviations d_i of the
+// reference c_i = k_i R with sum_i c_i = 6^D R and sum_i c_i c_i = 0): the exact sums rounded
+// once to FP64.
+//
+// Error-free extraction (Rump): adding and subtracting sigma = 1.5 2^(E + 4), where
+// |v_i| < 2^E, splits each value into a multiple q of 2^(E - 19) and a rest l below 2^(E - 20).
+// At most 27 q's add without rounding in FP32, and so do the l's as long as they are multiples
+// of 2^(E - 39), that is no value but zero is more than 15 binades below the largest; both
+// sums then meet in one FP64 addition.  Everything else (rare in a flow) goes through 64-bit
+// fixed point.  Returns false for a node that holds a value that is not finite.
+// The FP64 pipe takes 16 cycles per warp and SM for each instruction: 4 of them here, where
+// conversions and scalings took 12; the integer shifts of fixed point were 80 % of the rest.
+// Rsum = 6^D R in FP64 (exact).
+template <bool kDev>
+__device__ __forceinline__ bool exact_sums(const float (&v)[Q], float R, double Rsum, double &rho, double (&j)[3])
+{
+    float vmax = 0.0f;
+    uint32_t umin = 0xffffffffu; // of 2 bits - 1: zero wraps to the top
+#pragma unroll
+    for (int i = 0; i < Q; ++i) {
+        vmax = fmaxf(vmax, fabsf(v[i]));
+        umin = min(umin, 2u * __float_as_uint(v[i]) - 1u);
+    }
+    const int eb = int(__float_as_uint(vmax) >> 23), el = int((umin + 1u) >> 24);
+    bool nan = false;
+#pragma unroll
+    for (int i = 0; i < Q; ++i) nan = nan || v[i] != v[i]; // fmaxf drops NaN
+    if (!nan && eb >= 64 && eb < 192 && el >= eb - 15) {
+        const float sigma = __uint_as_float((uint32_t(eb + 5) << 23) | 0x400000u);
+        float q[Q], l[Q], rq, rl, jq[3], jl[3];
+#pragma unroll
+        for (int i = 0; i < Q; ++i) {
+            q[i] = (sigma + v[i]) - sigma;
+            l[i] = v[i] - q[i];
+        }
+        lattice_sums(q, rq, jq);
+        lattice_sums(l, rl, jl);
+        rho = f32_to_f64(rq) + f32_to_f64(rl);
+        if (kDev) rho += Rsum;
+#pragma unroll
+        for (int a = 0; a < D; ++a) j[a] = f32_to_f64(jq[a]) + f32_to_f64(jl[a]);
+        return true;
+    }
+    int emax = 1;
+#pragma unroll
+    for (int i = 0; i < Q; ++i) emax = max(emax, f32_expo(v[i]));
+    if (kDev) emax = max(emax, f32_expo(R) + 8); // 6^D R < 2^8 R
+    if (emax >= 255) return false;
+    const int E0 = emax - 33;
+    long long r = 0, jf[3] = {0, 0, 0};
+#pragma unroll
+    for (int i = 0; i < Q; ++i) {
+        const long long f = f32_fixed(v[i], E0);
+        r += f;
+#pragma unroll
+        for (int a = 0; a < D; ++a) {
+            if (vel(D, i, a) == 1) jf[a] += f;
+            if (vel(D, i, a) == -1) jf[a] -= f;
+        }
+    }
+    if (kDev) r += f32_fixed(R, E0) * (Q == 9 ? 36 : 216);
+    rho = fixed_to_f64(r, E0);
+#pragma unroll
+    for (int a = 0; a < D; ++a) j[a] = fixed_to_f64(jf[a], E0);
+    return true;
+}
+
+// 1 / rho to FP64 from the FP32 approximation r0 (relative error e < 2^-22): r0 (1 + e + e^2)
+__device__ __forceinline__ double rcp64(double rho)
+{
+    const float h = __double2float_rn(rho);
+    if (!(fabsf(h) > 1e-30f && fabsf(h) < 1e30f)) return 1.0 / rho;
+    const double r0 = f32_to_f64(rcp_(h)), e = fma(-rho, r0, 1.0);
+    return fma(r0, fma(e, e, e), r0);
+}
+
+// rho and u of the stored state (FP64) for the nodes n0 .. n0 + count - 1: FP64 storage in
+// FP64, the FP32-arithmetic storages by exact_sums (a node holding a value that is not finite
+// is summed in FP64).  4.8 M D3Q27 nodes of FP32 populations: 114 us = 5.9 TB/s (202 with
+// 64-bit fixed point for every value), FP32 deviations 133, FP16 131 (199); 8 M D2Q9 nodes 145,
+// 162, 162 (207, 237, 236; bound by the FP64 pipe).  At 48 registers (5 blocks of 256) rather than
+// the 80 the compiler takes: 141 us, too few loads in flight.
 template <class ST>
-__global__ void __launch_bounds__(kAuxBlock) k_moments(const typename ST::S *f,
-                                                      Geometry g, double rho0,
-                                                      double *rho_out,
-                                                      double *u_out, int64_t n0, int64_t count)
+__global__ void __launch_bounds__(kAuxBlock, 5) k_moments(const typename ST::S *f, Geometry g, float Rf, double Rsum,
+                                                      double *rho_out, double *u_out, int64_t n0, int64_t count)
 {
     wait_previous_kernel();
     const int64_t k = (int64_t)blockIdx.x * kAuxBlock + threadIdx.x;
     if (k >= count) return;
     const int64_t n = n0 + k;
-    const double R = double(dev_unit<D>(rho0));
     if constexpr (sizeof(typename ST::T) == 4) {
         float v[Q];
-        int emax = 1;
 #pragma unroll
-        for (int i = 0; i < Q; ++i) {
-            v[i] = ST::raw(f[(int64_t)i * g.N + n]);
-            emax = max(emax, f32_expo(v[i]));
-        }
-        const float Rf = dev_unit<D>(rho0);
-        if (ST::kDev) emax = max(emax, f32_expo(Rf) + 8); // 6^D R < 2^8 R
-        if (emax < 255) {
-            const int E0 = emax - 33;
-            long long r = 0, j[3] = {0, 0, 0};
-#pragma unroll
-            for (int i = 0; i < Q; ++i) {
-                const long long q = f32_fixed(v[i], E0);
-                r += q;
-#pragma unroll
-                for (int a = 0; a < D; ++a) {
-                    if (vel(D, i, a) == 1) j[a] += q;
-                    if (vel(D, i, a) == -1) j[a] -= q;
-                }
-            }
-            if (ST::kDev) r += f32_fixed(Rf, E0) * (Q == 9 ? 36 : 216);
-            const double rho = fixed_to_f64(r, E0);
+        for (int i = 0; i < Q; ++i) v[i] = ST::raw(f[(int64_t)i * g.N + n]);
+        double rho, j[3];
+        if (exact_sums<ST::kDev>(v, Rf, Rsum, rho, j)) {
             if (rho_out) rho_out[n] = rho;
             if (u_out) {
-                const double ir = 1.0 / rho;
+                const double ir = rcp64(rho);
 #pragma unroll
-                for (int a = 0; a < D; ++a) u_out[(int64_t)a * g.N + n] = fixed_to_f64(j[a], E0) * ir;
+                for (int a = 0; a < D; ++a) u_out[(int64_t)a * g.N + n] = j[a] * ir;
             }
             return;
         }
@@ -461,7 +618,7 @@ __global__ void __launch_bounds__(kAuxBlock) k_moments(const typename ST::S *f,
     double r = 0.0, j[3] = {0.0, 0.0, 0.0};
 #pragma unroll
     for (int i = 0; i < Q; ++i) {
-        const double v = ST::load64(f[(int64_t)i * g.N + n], weight_k(D, i) * R);
+        const double v = ST::load64(f[(int64_t)i * g.N + n], weight_k(D, i) * double(Rf));
         r += v;
 #pragma unroll
         for (int a = 0; a < D; ++a) j[a] += vel(D, i, a) * v;
@@ -1083,22 +1240,60 @@ __global__ void __launch_bounds__(kAuxBlock) k_step_adjoint(const typename ST::S
 }
 
 // Kinetic energy L = 1/2 sum rho |u|^2 of a stored field (FP64 sum into acc[0])
-// and, optionally, its gradient dL/df_i = c_i . u - |u|^2 / 2.
+// and, optionally, its gradient dL/df_i = c_i . u - |u|^2 / 2.  The FP32-arithmetic storages
+// take rho and rho u from exact_sums and form the gradient in double-float, rounded once to
+// FP32: 4.8 M D3Q27 nodes with gradient 207 us, where FP64 sums and gradients kept the FP64
+// pipe busy for 2.38 ms; 137 k nodes 15 (84), 65 k D2Q9 nodes 11 (26).
 template <class ST>
-__global__ void __launch_bounds__(kAuxBlock) k_kinetic_energy(const typename ST::S *__restrict__ f,
-                                                             Geometry g, double rho0, double *__restrict__ acc,
-                                                             typename ST::T *__restrict__ grad)
+__global__ void __launch_bounds__(kAuxBlock, 4) k_kinetic_energy(const typename ST::S *f, Geometry g, float Rf, double Rsum,
+                                                             double *__restrict__ acc, typename ST::T *grad)
 {
     wait_previous_kernel();
     using T = typename ST::T;
     double e = 0.0;
-    const double R = double(dev_unit<D>(rho0));
     for (int64_t n = (int64_t)blockIdx.x * kAuxBlock + threadIdx.x; n < g.N; n += (int64_t)gridDim.x * kAuxBlock) {
         double r = 0.0, j[3] = {0.0, 0.0, 0.0};
+        if constexpr (sizeof(T) == 4) {
+            float v[Q];
+#pragma unroll
+            for (int i = 0; i < Q; ++i) v[i] = ST::raw(f[(int64_t)i * g.N + n]);
+            if (exact_sums<ST::kDev>(v, Rf, Rsum, r, j)) {
+                const double ir = rcp64(r);
+                double uu = 0.0, u[3];
+#pragma unroll
+                for (int a = 0; a < D; ++a) {
+                    u[a] = j[a] * ir;
+                    uu = fma(u[a], u[a], uu);
+                }
+                e = fma(0.5 * r, uu, e);
+                if (grad) {
+                    DF ud[3], base = df_mulf(df_from_double(uu), -0.5f);
+#pragma unroll
+                    for (int a = 0; a < D; ++a) ud[a] = df_from_double(u[a]);
+                    auto along = [](DF b, DF w, int c) { return c == 0 ? b : df_add(b, c > 0 ? w : df_neg(w)); };
+#pragma unroll
+                    for (int x = 0; x < 3; ++x) {
+                        const DF bx = along(base, ud[0], x - 1);
+#pragma unroll
+                        for (int y = 0; y < 3; ++y) {
+                            const DF by = along(bx, ud[1], y - 1);
+                            if constexpr (D == 2) {
+                                grad[(int64_t)(3 * x + y) * g.N + n] = by.hi;
+                            } else {
+#pragma unroll
+                                for (int z = 0; z < 3; ++z)
+                                    grad[(int64_t)(9 * x + 3 * y + z) * g.N + n] = along(by, ud[2], z - 1).hi;
+                            }
+                        }
+                    }
+                }
+                continue;
+            }
+        }
         double fv[Q];
 #pragma unroll
         for (int i = 0; i < Q; ++i) {
-            fv[i] = ST::load64(ld_pop<true>(f + (int64_t)i * g.N + n), weight_k(D, i) * R);
+            fv[i] = ST::load64(f[(int64_t)i * g.N + n], weight_k(D, i) * double(Rf));
             r += fv[i];
 #pragma unroll
             for (int a = 0; a < D; ++a) j[a] += vel(D, i, a) * fv[i];
@@ -1120,8 +1315,14 @@ __global__ void __launch_bounds__(kAuxBlock) k_kinetic_energy(const typename ST:
             }
         }
     }
+    __shared__ double s_e[kAuxBlock / 32];
     e = warp_sum(e);
-    if ((threadIdx.x & 31) == 0) atomicAdd(acc, e);
+    if ((threadIdx.x & 31) == 0) s_e[threadIdx.x >> 5] = e;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int w = 1; w < kAuxBlock / 32; ++w) e += s_e[w];
+        atomicAdd(acc, e);
+    }
 }
 
 // Derivatives of f = f^eq(rho, u) (the initial state) with respect to rho and u:
@@ -1458,8 +1659,10 @@ cudaError_t ELBM_CAT(launch_kinetic_energy, ELBM_SUFFIX)(int storage, const void
     unsigned blocks = blocks_for(g.N, kAuxBlock);
     const unsigned cap = unsigned(num_sms > 0 ? num_sms : 1) * 8u;
     if (blocks > cap) blocks = cap;
+    const float Rf = dev_unit<D>(rho0);
+    const double Rsum = (Q == 9 ? 36.0 : 216.0) * double(Rf);
     ELBM_STORAGE_SWITCH(storage, return launch(k_kinetic_energy<ST>, blocks, kAuxBlock, s,
-                                               static_cast<const typename ST::S *>(f), g, rho0, acc,
+                                               static_cast<const typename ST::S *>(f), g, Rf, Rsum, acc,
                                                static_cast<typename ST::T *>(grad)))
     return cudaGetLastError();
 }
@@ -1495,8 +1698,10 @@ cudaError_t ELBM_CAT(launch_moments, ELBM_SUFFIX)(int storage, const void *f, co
 {
     using namespace ELBM_SUFFIX;
     if (count <= 0) return cudaSuccess;
+    const float Rf = dev_unit<D>(rho0);
+    const double Rsum = (Q == 9 ? 36.0 : 216.0) * double(Rf);
     ELBM_STORAGE_SWITCH(storage, return launch(k_moments<ST>, blocks_for(count, kAuxBlock), kAuxBlock, s,
-                                               static_cast<const typename ST::S *>(f), g, rho0, rho_out,
+                                               static_cast<const typename ST::S *>(f), g, Rf, Rsum, rho_out,
                                                u_out, n0, count))
     return cudaGetLastError();
 }
