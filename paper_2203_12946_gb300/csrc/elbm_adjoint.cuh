@@ -8,6 +8,9 @@
 // Membership in Omega+ / Omega- is held fixed (each restricted term is O(x^3),
 // so the sums are twice differentiable across x = 0); the cutoff and the clamp
 // are branches, differentiated on the side the forward pass took.
+//
+// node_vjp is the general form (FP64, and FP32 nodes whose |x|max is beyond the power
+// series); node_vjp_series the FP32 form of all other nodes, which is what a flow has.
 #pragma once
 
 #include "elbm_device.cuh"
@@ -324,6 +327,289 @@ __device__ void node_vjp(const T (&F)[Lattice<D>::Q], const T (&gin0)[Lattice<D>
     feq_vjp(gin, V);
 #pragma unroll
     for (int i = 0; i < Q; ++i) h[i] = gin[i] + beta * (s * Fb[i] + alpha * (V[i] - gin[i]));
+}
+
+// ---------------------------------------------------------------------------
+// FP32 vector-Jacobian product of one node's collision where |x|max < 0.04.
+//
+// There alpha depends on the populations through the power sums M_k = <f, x^k> and, over
+// Omega-, S_k alone (node_collide_pairs), so with the adjoints m_k and s_k of the sums
+//   P(x) = sum_k m_k x^k + [x < 0] sum_k s_k x^k,   d alpha / d f_i = P(x_i) + f_i P'(x_i) dx_i/df_i + ...,
+// and as x_i = feq_i / f_i - 1 the derivative with respect to f_i at fixed feq is
+//   q_i = P(x_i) - (1 + x_i) P'(x_i),
+// and that with respect to feq_i is P'(x_i): no division per population.  The VJP of feq is
+// linear, so the whole product needs it once, applied to l_i = s P'(x_i) + alpha g_i with
+// s = <g, feq - f>:
+//   h_j = g_j + beta (s q_j - alpha g_j + V(l)_j).
+// V is separable: per axis a line (l_-, l_0, l_+) with d = l_+ - l_-, w = 2 (l_+ + l_-) - 4 l_0
+// contracts with 1 + eps to (l_+ + l_- + 4 l_0) + 3u d + t w, and with d eps / du to
+// 3 d + (3u/s) w (eps = -t, 2t -+ 3u; the weights' 4 for the rest component included), so that
+// 1 + eps is never rounded, and
+//   V_j = 6^-D (C_0 + sum_a C_a (c_ja - u_a)),
+// C_0 the full contraction and C_a the one with axis a differentiated: 160 operations where
+// the products written out per population take over 1000.
+// ---------------------------------------------------------------------------
+struct AxisVjp {
+    float u, t, v; // velocity, t = sqrt(1 + 3u^2) - 1, v = 3u / sqrt(1 + 3u^2)
+};
+__device__ __forceinline__ AxisVjp axis_vjp(float u)
+{
+    const float uu3 = 3.0f * u * u, s = sqrt_(1.0f + uu3);
+    return {u, div_(uu3, 1.0f + s), 3.0f * u * rcp_(s)};
+}
+// One line along an axis against 1 + eps (returned) and against d eps / du (*du, may be null).
+__device__ __forceinline__ float line_vjp(float lm, float l0, float lp, const AxisVjp &a, float *du)
+{
+    const float c0 = 4.0f * l0, d = lp - lm, sg = lp + lm, w = fmaf(2.0f, sg, -c0);
+    if (du) *du = fmaf(3.0f, d, a.v * w);
+    return (sg + c0) + fmaf(3.0f * a.u, d, a.t * w);
+}
+// C[0] = sum_i l_i k_i prod (1 + eps), C[1 + a] with axis a differentiated.
+template <int D>
+__device__ __forceinline__ void feq_contract(const float (&l)[Lattice<D>::Q], const AxisVjp (&ax)[D], float (&C)[D + 1])
+{
+    constexpr int P = Lattice<D>::Q / 3;
+    float A[P], Ad[P]; // contracted along the last axis
+#pragma unroll
+    for (int k = 0; k < P; ++k) A[k] = line_vjp(l[3 * k], l[3 * k + 1], l[3 * k + 2], ax[D - 1], &Ad[k]);
+    if constexpr (D == 2) {
+        C[0] = line_vjp(A[0], A[1], A[2], ax[0], &C[1]);
+        C[2] = line_vjp(Ad[0], Ad[1], Ad[2], ax[0], nullptr);
+    } else {
+        float B[3], By[3], Bz[3];
+#pragma unroll
+        for (int x = 0; x < 3; ++x) {
+            B[x] = line_vjp(A[3 * x], A[3 * x + 1], A[3 * x + 2], ax[1], &By[x]);
+            Bz[x] = line_vjp(Ad[3 * x], Ad[3 * x + 1], Ad[3 * x + 2], ax[1], nullptr);
+        }
+        C[0] = line_vjp(B[0], B[1], B[2], ax[0], &C[1]);
+        C[2] = line_vjp(By[0], By[1], By[2], ax[0], nullptr);
+        C[D] = line_vjp(Bz[0], Bz[1], Bz[2], ax[0], nullptr);
+    }
+}
+// V_j = base + sum_a c_ja step_a of the contraction C (6^-D in two parts).
+template <int D>
+__device__ __forceinline__ void feq_vjp_terms(const float (&C)[D + 1], const AxisVjp (&ax)[D], float &base, float (&step)[D])
+{
+    constexpr float W = float(weight_unit(D)), Wl = weight_unit_lo<D, float>();
+    base = fmaf(C[0], W, C[0] * Wl);
+#pragma unroll
+    for (int a = 0; a < D; ++a) {
+        step[a] = fmaf(C[1 + a], W, C[1 + a] * Wl);
+        base = fmaf(-step[a], ax[a].u, base);
+    }
+}
+// The positive root of quad_root with its partial derivatives, scaled by b alike.
+__device__ __forceinline__ RootGrad<float> root_grad_scaled(float a, float b, float c)
+{
+    const float rb = rcp_(b), q = c * rb, p = a * rb;
+    const float w = sqrt_(fmaf(-4.0f * p, q, 1.0f)), rd = rcp_(1.0f + w), k = 4.0f * q * rd * rd * rcp_(w);
+    const float dq = fmaf(k, p, 2.0f * rd), dp = k * q;
+    return {2.0f * q * rd, dp * rb, -(q * dq + p * dp) * rb, dq * rb};
+}
+
+// F: populations, g: dL/df*; h receives dL/dF.  Returns false (h untouched) where the node
+// needs node_vjp.  kForce as in node_vjp.
+template <int D, bool kForce = false>
+__device__ __forceinline__ bool node_vjp_series(const float (&F)[Lattice<D>::Q], float (&g)[Lattice<D>::Q],
+                                                const CollideParams &p, float (&h)[Lattice<D>::Q], float *dforce = nullptr)
+{
+    constexpr int Q = Lattice<D>::Q, NP = Pairs<D>::NP;
+    const float beta = p.beta_f;
+    // moments from the deviations F_i - k_i W (as node_collide)
+    float drho, j[D];
+    {
+        float s0[Q / 3], s1[Q / 3];
+#pragma unroll
+        for (int k = 0; k < Q / 3; ++k) {
+            float d[3];
+#pragma unroll
+            for (int c = 0; c < 3; ++c) d[c] = F[3 * k + c] - float(weight_k(D, 3 * k + c)) * float(weight_unit(D));
+            s0[k] = (d[0] + d[2]) + d[1];
+            s1[k] = d[2] - d[0];
+        }
+        if constexpr (D == 2) {
+            drho = s0[0] + s0[1] + s0[2];
+            j[0] = s0[2] - s0[0];
+            j[1] = s1[0] + s1[1] + s1[2];
+        } else {
+            float t[3], ty[3], tz[3];
+#pragma unroll
+            for (int a = 0; a < 3; ++a) {
+                t[a] = s0[3 * a] + s0[3 * a + 1] + s0[3 * a + 2];
+                ty[a] = s0[3 * a + 2] - s0[3 * a];
+                tz[a] = s1[3 * a] + s1[3 * a + 1] + s1[3 * a + 2];
+            }
+            drho = t[0] + t[1] + t[2];
+            j[0] = t[2] - t[0];
+            j[1] = ty[0] + ty[1] + ty[2];
+            j[D - 1] = tz[0] + tz[1] + tz[2];
+        }
+    }
+    drho -= float(double(Q == 9 ? 36 : 216) * double(weight_unit_lo<D, float>()));
+    const float rho = 1.0f + drho, irho = rcp_nr(rho);
+    const float r = fmaf(rho, float(weight_unit(D)), rho * weight_unit_lo<D, float>());
+    AxisVjp ax[D];
+    float eps[D][3];
+#pragma unroll
+    for (int a = 0; a < D; ++a) {
+        ax[a] = axis_vjp(j[a] * irho);
+        eps[a][0] = fmaf(-3.0f, ax[a].u, 2.0f * ax[a].t);
+        eps[a][1] = -ax[a].t;
+        eps[a][2] = fmaf(3.0f, ax[a].u, 2.0f * ax[a].t);
+    }
+    // departures, in pairs (node_collide_pairs)
+    float2 f[NP], x[NP];
+    float xabs = 0.0f;
+#pragma unroll
+    for (int k = 0; k < NP; ++k) {
+        const int m = pair_axis(D, k), i0 = pair_pop(D, k, 0), i1 = pair_pop(D, k, 1);
+        f[k] = f2(F[i0], i1 >= 0 ? F[i1] : 1.0f);
+        float G = 0.0f;
+        bool first = true;
+#pragma unroll
+        for (int a = 0; a < D; ++a) {
+            if (a == m) continue;
+            const float e = eps[a][vel(D, i0, a) + 1];
+            G = first ? e : G + e + G * e;
+            first = false;
+        }
+        float2 E = f2(G, 0.0f);
+        if (m >= 0) {
+            const float2 em = f2(eps[m][0], eps[m][2]);
+            E = pfma(f2(G), em, padd(f2(G), em));
+        }
+        const float2 kr = pmul(f2(kpair<D>(k, 0), kpair<D>(k, 1)), f2(r));
+        float2 delta = pfma(kr, E, psub(kr, f[k]));
+        if (m < 0) delta.y = 0.0f; // padding lane
+        x[k] = pmul(delta, prcp(f[k]));
+        xabs = fmaxf(xabs, fmaxf(fabsf(x[k].x), fabsf(x[k].y)));
+    }
+    const bool lbgk = p.mode == kModeLBGK;
+    if (!lbgk && !(xabs < 0.04f)) return false;
+
+    if constexpr (kForce) {
+        // g <- (I + dPhi/df*)^T g, Phi the body-force term, and d<g, C + Phi>/dF_b
+        AxisVjp av[D];
+#pragma unroll
+        for (int a = 0; a < D; ++a) av[a] = axis_vjp(fmaf(float(p.force[a]), irho, ax[a].u));
+        float Cu[D + 1], Cv[D + 1], bu, bv, su[D], sv[D];
+        feq_contract<D>(g, ax, Cu);
+        feq_contract<D>(g, av, Cv);
+        feq_vjp_terms<D>(Cu, ax, bu, su);
+        feq_vjp_terms<D>(Cv, av, bv, sv);
+#pragma unroll
+        for (int i = 0; i < Q; ++i) {
+            float d = bv - bu;
+#pragma unroll
+            for (int a = 0; a < D; ++a) d += float(vel(D, i, a)) * (sv[a] - su[a]);
+            g[i] += d;
+        }
+        if (dforce) {
+#pragma unroll
+            for (int a = 0; a < D; ++a) dforce[a] += sv[a]; // G_a / rho: d v_a / d F_b,a = 1 / rho
+        }
+    }
+
+    // alpha and the adjoints m_k, s_k of the power sums
+    float alpha = 2.0f, m2 = 0.0f, m3 = 0.0f, m4 = 0.0f, m5 = 0.0f, m6 = 0.0f, s3 = 0.0f, s4 = 0.0f, s5 = 0.0f, s6 = 0.0f;
+    if (!lbgk && !(p.cutoff && xabs < float(kCutoff))) {
+        float2 M2 = f2(0.0f), M3 = f2(0.0f), M4 = f2(0.0f), M5 = f2(0.0f), M6 = f2(0.0f);
+        float2 A3 = f2(0.0f), A4 = f2(0.0f), A5 = f2(0.0f), A6 = f2(0.0f);
+#pragma unroll
+        for (int k = 0; k < NP; ++k) {
+            const float2 x2 = pmul(x[k], x[k]), g2 = pmul(f[k], x2), g4 = pmul(g2, x2);
+            const float2 axk = f2(fabsf(x[k].x), fabsf(x[k].y)), xax = pmul(x[k], axk);
+            M2 = padd(M2, g2), M3 = pfma(g2, x[k], M3), M4 = padd(M4, g4), M5 = pfma(g4, x[k], M5), M6 = pfma(g4, x2, M6);
+            A3 = pfma(g2, axk, A3), A4 = pfma(g2, xax, A4), A5 = pfma(g4, axk, A5), A6 = pfma(g4, xax, A6);
+        }
+        const float S2 = M2.x + M2.y, T3 = M3.x + M3.y, T4 = M4.x + M4.y, T5 = M5.x + M5.y, T6 = M6.x + M6.y;
+        const float S3 = 0.5f * (T3 - (A3.x + A3.y)), S4 = 0.5f * (T4 - (A4.x + A4.y));
+        const float S5 = 0.5f * (T5 - (A5.x + A5.y)), S6 = 0.5f * (T6 - (A6.x + A6.y));
+        const float b1 = 0.5f * S2;
+        const float c1 = S2 + fmaf(T3, -0.5f, fmaf(T4, 0.25f, fmaf(T5, -0.125f, T6 * 0.0625f)));
+        const float c = S2 + fmaf(T3, -0.5f, fmaf(T4, 1.0f / 3.0f, fmaf(T5, -0.25f, T6 * 0.2f)));
+        if (b1 > 0.0f) {
+            const RootGrad<float> rl = root_grad_scaled(0.5f * S3, b1, c1); // alpha_Lower
+            float aLb = 1.0f, b1b = 0.0f, cb = 0.0f, Pb = 0.0f, kk = 0.0f;
+            alpha = rl.r;
+            if (p.mode != kModeLower) {
+                const float bb2 = beta * beta, kap = (2.0f / 15.0f) * bb2;
+                kk = p.b_variant ? rl.r : rl.r * beta;
+                const float P3 = T3 - S3, P4 = T4 - S4, P5 = T5 - S5, P6 = T6 - S6;
+                const float bsum = fmaf(kk, fmaf(kk, fmaf(kk, -0.25f * P6, 0.375f * P5), -0.625f * P4), 1.25f * P3);
+                const float b = fmaf(-kap * rl.r, bsum, b1);
+                const RootGrad<float> rh = root_grad_scaled(bb2 * (1.0f / 6.0f) * S3, b, c); // h
+                const float hb = rh.r * beta;
+                const float A = bb2 * fmaf(hb, fmaf(hb, fmaf(hb, -0.2f * S6, 0.05f * S5), (-1.0f / 12.0f) * S4),
+                                           (1.0f / 6.0f) * S3);
+                const RootGrad<float> ra = root_grad_scaled(A, b, c); // alpha_Higher
+                alpha = ra.r;
+                const float Ab = ra.ra * bb2;
+                const float hbar = Ab * beta * fmaf(hb, fmaf(hb, -0.6f * S6, 0.1f * S5), (-1.0f / 12.0f) * S4);
+                s3 = Ab * (1.0f / 6.0f) + hbar * rh.ra * bb2 * (1.0f / 6.0f);
+                s4 = Ab * hb * (-1.0f / 12.0f);
+                s5 = Ab * hb * hb * 0.05f;
+                s6 = Ab * hb * hb * hb * -0.2f;
+                const float bbar = fmaf(hbar, rh.rb, ra.rb);
+                cb = fmaf(hbar, rh.rc, ra.rc);
+                b1b = bbar;
+                Pb = -bbar * kap * rl.r; // adjoint of bsum
+                const float kb = Pb * fmaf(kk, fmaf(kk, -0.75f * P6, 0.75f * P5), -0.625f * P4);
+                aLb = fmaf(-bbar * kap, bsum, kb * (p.b_variant ? 1.0f : beta));
+            }
+            s3 = fmaf(aLb * 0.5f, rl.ra, s3);
+            b1b = fmaf(aLb, rl.rb, b1b);
+            const float c1b = aLb * rl.rc;
+            const float P3b = 1.25f * Pb, P4b = -0.625f * kk * Pb, P5b = 0.375f * kk * kk * Pb, P6b = -0.25f * kk * kk * kk * Pb;
+            m2 = 0.5f * b1b + c1b + cb;
+            m3 = P3b - 0.5f * (c1b + cb);
+            m4 = P4b + 0.25f * c1b + (1.0f / 3.0f) * cb;
+            m5 = P5b - 0.125f * c1b - 0.25f * cb;
+            m6 = P6b + 0.0625f * c1b + 0.2f * cb;
+            s3 -= P3b, s4 -= P4b, s5 -= P5b, s6 -= P6b;
+        }
+    }
+    // s = <g, feq - f>; then l = s P'(x) + alpha g, and q in the place of x
+    float2 sp = f2(0.0f);
+#pragma unroll
+    for (int k = 0; k < NP; ++k) {
+        const int i0 = pair_pop(D, k, 0), i1 = pair_pop(D, k, 1);
+        sp = pfma(f2(g[i0], i1 >= 0 ? g[i1] : 0.0f), pmul(x[k], f[k]), sp);
+    }
+    const float s = sp.x + sp.y;
+    float l[Q];
+#pragma unroll
+    for (int k = 0; k < NP; ++k) {
+        const int i0 = pair_pop(D, k, 0), i1 = pair_pop(D, k, 1);
+        const float2 xk = x[k], xm = f2(fminf(xk.x, 0.0f), fminf(xk.y, 0.0f));
+        const float2 x2 = pmul(xk, xk), xm2 = pmul(xm, xm);
+        const float2 pm = pfma(pfma(pfma(pfma(f2(m6), xk, f2(m5)), xk, f2(m4)), xk, f2(m3)), xk, f2(m2));
+        const float2 ps = pfma(pfma(pfma(f2(s6), xm, f2(s5)), xm, f2(s4)), xm, f2(s3));
+        const float2 P = pfma(x2, pm, pmul(pmul(xm2, xm), ps));
+        const float2 dm = pfma(pfma(pfma(pfma(f2(6.0f * m6), xk, f2(5.0f * m5)), xk, f2(4.0f * m4)), xk, f2(3.0f * m3)), xk,
+                               f2(2.0f * m2));
+        const float2 ds = pfma(pfma(pfma(f2(6.0f * s6), xm, f2(5.0f * s5)), xm, f2(4.0f * s4)), xm, f2(3.0f * s3));
+        const float2 lam = pfma(xk, dm, pmul(xm2, ds));
+        x[k] = pfma(lam, psub(f2(-1.0f), xk), P); // q
+        const float2 lk = pfma(f2(s), lam, pmul(f2(alpha), f2(g[i0], i1 >= 0 ? g[i1] : 0.0f)));
+        l[i0] = lk.x;
+        if (i1 >= 0) l[i1] = lk.y;
+    }
+    float C[D + 1], base, step[D];
+    feq_contract<D>(l, ax, C);
+    feq_vjp_terms<D>(C, ax, base, step);
+#pragma unroll
+    for (int i = 0; i < Q; ++i) {
+        float V = base;
+#pragma unroll
+        for (int a = 0; a < D; ++a)
+            if (vel(D, i, a)) V = vel(D, i, a) > 0 ? V + step[a] : V - step[a];
+        const int sl = pair_slot(D, i);
+        const float q = (sl & 1) ? x[sl >> 1].y : x[sl >> 1].x;
+        h[i] = fmaf(beta, fmaf(s, q, fmaf(-alpha, g[i], V)), g[i]);
+    }
+    return true;
 }
 
 } // namespace eelbm

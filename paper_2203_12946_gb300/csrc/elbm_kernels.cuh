@@ -1191,39 +1191,97 @@ __global__ void __launch_bounds__(BX / nodes_per_thread<D, ST>()) k_step_persist
 // the transpose of pull streaming sends h_i(x) to node x - c_i (a push).
 // Gradient arrays are SoA [Q][N] in the compute type.
 // --------------------------------------------------------------------------
-template <class ST, bool kForce = false>
-__global__ void __launch_bounds__(kAuxBlock) k_step_adjoint(const typename ST::S *__restrict__ fin,
-                                                           const typename ST::T *__restrict__ gnext,
-                                                           typename ST::T *__restrict__ gout, Geometry g,
-                                                           CollideParams p, double *__restrict__ dforce)
+// FP32: nodes on the power series (node_vjp_series); the others go through node_vjp, kept
+// out of line so that its registers do not bound the kernel's occupancy.
+template <bool kForce>
+__device__ __noinline__ void node_vjp_general(const float (&F)[Q], const float (&g)[Q], const CollideParams &p, float (&h)[Q],
+                                              float *dforce)
+{
+    node_vjp<D, float, kForce>(F, g, p, h, dforce);
+}
+
+template <class ST>
+constexpr int adjoint_block()
+{
+    return sizeof(typename ST::T) == 4 ? 128 : kAuxBlock;
+}
+template <class ST, int kAddr, bool kForce = false>
+__global__ void __launch_bounds__(adjoint_block<ST>(), sizeof(typename ST::T) == 4 ? 4 : 1)
+    k_step_adjoint(const typename ST::S *__restrict__ fin, const typename ST::T *__restrict__ gnext,
+                   typename ST::T *__restrict__ gout, Geometry g, CollideParams p, RowDiv rd, double *__restrict__ dforce)
 {
     wait_previous_kernel();
     using T = typename ST::T;
-    const int64_t n = (int64_t)blockIdx.x * kAuxBlock + threadIdx.x;
+    using S = typename ST::S;
+    constexpr int kBlock = adjoint_block<ST>();
     T dfl[3] = {T(0), T(0), T(0)};
-    if (n < g.N) {
-        int x, y, z;
-        node_coords(n, g, x, y, z);
-        T F[Q], gl[Q], h[Q];
-        pull_load<D, ST>(fin, g, x, y, z, p.dunit_f, F);
+    T F[Q], gl[Q], h[Q];
+    // J^T g of the node
+    auto vjp = [&]() {
+        if constexpr (sizeof(T) == 4) {
+            if (!node_vjp_series<D, kForce>(F, gl, p, h, dfl)) {
+                float Fm[Q], gm[Q], hm[Q], dm[3] = {0.0f, 0.0f, 0.0f}; // in memory for the call; the rest stays in registers
 #pragma unroll
-        for (int i = 0; i < Q; ++i) gl[i] = __ldcs(gnext + (int64_t)i * g.N + n);
-        node_vjp<D, T, kForce>(F, gl, p, h, dfl);
-        const int xm = x == 0 ? g.nx - 1 : x - 1, xp = x == g.nx - 1 ? 0 : x + 1;
-        const int ym = y == 0 ? g.ny - 1 : y - 1, yp = y == g.ny - 1 ? 0 : y + 1;
-        const int zm = z == 0 ? g.nz - 1 : z - 1, zp = z == g.nz - 1 ? 0 : z + 1;
+                for (int i = 0; i < Q; ++i) Fm[i] = F[i], gm[i] = gl[i];
+                node_vjp_general<kForce>(Fm, gm, p, hm, dm);
 #pragma unroll
-        for (int i = 0; i < Q; ++i) {
-            const int cx = vel(D, i, 0), cy = vel(D, i, 1), cz = D == 3 ? vel(D, i, 2) : 0;
-            const int dx = cx == 1 ? xm : (cx == -1 ? xp : x);
-            const int dy = cy == 1 ? ym : (cy == -1 ? yp : y);
-            const int dz = cz == 1 ? zm : (cz == -1 ? zp : z);
-            gout[(int64_t)i * g.N + ((int64_t)dz * g.ny + dy) * g.nx + dx] = h[i];
+                for (int i = 0; i < Q; ++i) h[i] = hm[i];
+#pragma unroll
+                for (int a = 0; a < 3; ++a) dfl[a] += dm[a];
+            }
+        } else {
+            node_vjp<D, T, kForce>(F, gl, p, h, dfl);
+        }
+    };
+    if constexpr (kAddr == kAddrBytes) {
+        // as k_step: consecutive nodes of an xy-plane, byte offsets; the push of h_i goes where
+        // the pull of f_i came from
+        const uint32_t nx = uint32_t(g.nx), ny = uint32_t(g.ny), nz = uint32_t(g.nz), N = uint32_t(g.N);
+        const uint32_t plane = nx * ny, xy = blockIdx.x * kBlock + threadIdx.x, z = blockIdx.y;
+        if (xy < plane) {
+            const uint32_t y = div_row(xy, rd), x = xy - y * nx;
+            const uint32_t sx[3] = {x == nx - 1 ? 0 : x + 1, x, x == 0 ? nx - 1 : x - 1};
+            const uint32_t sy[3] = {y == ny - 1 ? 0 : (y + 1) * nx, y * nx, (y == 0 ? ny - 1 : y - 1) * nx};
+            const uint32_t sz[3] = {z == nz - 1 ? 0 : z + 1, z, z == 0 ? nz - 1 : z - 1};
+            auto src = [&](int i, uint32_t B) {
+                const int cx = vel(D, i, 0), cy = vel(D, i, 1), cz = D == 3 ? vel(D, i, 2) : 0;
+                return (sy[cy + 1] + sx[cx + 1]) * B + (uint32_t(i) * N + sz[cz + 1] * plane) * B;
+            };
+#pragma unroll
+            for (int i = 0; i < Q; ++i)
+                F[i] = ST::load(ld_pop<true>(at<kAddrBytes>(fin, src(i, sizeof(S)))), dev_ref<D, T>(i, p.dunit_f));
+            const uint32_t n = (z * plane + xy) * uint32_t(sizeof(T));
+#pragma unroll
+            for (int i = 0; i < Q; ++i) gl[i] = __ldcs(at<kAddrBytes>(gnext, uint32_t(i) * N * uint32_t(sizeof(T)) + n));
+            vjp();
+#pragma unroll
+            for (int i = 0; i < Q; ++i) *at<kAddrBytes>(gout, src(i, sizeof(T))) = h[i];
+        }
+    } else {
+        const int64_t n = (int64_t)blockIdx.x * kBlock + threadIdx.x;
+        if (n < g.N) {
+            int x, y, z;
+            node_coords(n, g, x, y, z);
+            pull_load<D, ST>(fin, g, x, y, z, p.dunit_f, F);
+#pragma unroll
+            for (int i = 0; i < Q; ++i) gl[i] = __ldcs(gnext + (int64_t)i * g.N + n);
+            vjp();
+            const int xm = x == 0 ? g.nx - 1 : x - 1, xp = x == g.nx - 1 ? 0 : x + 1;
+            const int ym = y == 0 ? g.ny - 1 : y - 1, yp = y == g.ny - 1 ? 0 : y + 1;
+            const int zm = z == 0 ? g.nz - 1 : z - 1, zp = z == g.nz - 1 ? 0 : z + 1;
+#pragma unroll
+            for (int i = 0; i < Q; ++i) {
+                const int cx = vel(D, i, 0), cy = vel(D, i, 1), cz = D == 3 ? vel(D, i, 2) : 0;
+                const int dx = cx == 1 ? xm : (cx == -1 ? xp : x);
+                const int dy = cy == 1 ? ym : (cy == -1 ? yp : y);
+                const int dz = cz == 1 ? zm : (cz == -1 ? zp : z);
+                gout[(int64_t)i * g.N + ((int64_t)dz * g.ny + dy) * g.nx + dx] = h[i];
+            }
         }
     }
     if constexpr (kForce) {
         // d/dF_b summed over the block (FP64), one atomic per block and component
-        __shared__ double s_df[kAuxBlock / 32][3];
+        __shared__ double s_df[kBlock / 32][3];
         const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 #pragma unroll
         for (int a = 0; a < D; ++a) {
@@ -1233,7 +1291,7 @@ __global__ void __launch_bounds__(kAuxBlock) k_step_adjoint(const typename ST::S
         __syncthreads();
         if (dforce && threadIdx.x < D) {
             double v = 0.0;
-            for (int w = 0; w < kAuxBlock / 32; ++w) v += s_df[w][threadIdx.x];
+            for (int w = 0; w < kBlock / 32; ++w) v += s_df[w][threadIdx.x];
             atomicAdd(&dforce[threadIdx.x], v);
         }
     }
@@ -1637,18 +1695,39 @@ cudaError_t ELBM_CAT(launch_step_adjoint, ELBM_SUFFIX)(int storage, const void *
     using namespace ELBM_SUFFIX;
     if (g.N == 0) return cudaSuccess;
     const bool forced = dforce || p.force[0] != 0.0 || p.force[1] != 0.0 || p.force[2] != 0.0;
-    if (forced) {
-        ELBM_STORAGE_SWITCH(storage, return launch(k_step_adjoint<ST, true>, blocks_for(g.N, kAuxBlock),
-                                                   kAuxBlock, s, static_cast<const typename ST::S *>(fin),
-                                                   static_cast<const typename ST::T *>(gnext),
-                                                   static_cast<typename ST::T *>(gout), g, p, dforce))
-    } else {
-        ELBM_STORAGE_SWITCH(storage, return launch(k_step_adjoint<ST>, blocks_for(g.N, kAuxBlock), kAuxBlock,
-                                                   s, static_cast<const typename ST::S *>(fin),
-                                                   static_cast<const typename ST::T *>(gnext),
-                                                   static_cast<typename ST::T *>(gout), g, p, nullptr))
+    // byte offsets where the gradient (and so the state) fills less than 2^32 bytes; FP64, bound
+    // by its arithmetic, keeps the 1D grid
+    const bool bytes = storage != ELBM_STORE_F64 && uint64_t(Q) * uint64_t(g.N) * 4u <= 0xffffffffull && g.nz <= 65535;
+    const int64_t plane = int64_t(g.nx) * g.ny;
+    const RowDiv rd = row_div(uint32_t(g.nx));
+#define ELBM_ADJOINT(ADDR, FORCE, GRID)                                                                \
+    return launch(k_step_adjoint<ST, ADDR, FORCE>, GRID, adjoint_block<ST>(), s,                       \
+                  static_cast<const typename ST::S *>(fin), static_cast<const typename ST::T *>(gnext), \
+                  static_cast<typename ST::T *>(gout), g, p, rd, dforce)
+    if (storage == ELBM_STORE_F64) {
+        using ST = StoreF64;
+        if (forced) ELBM_ADJOINT(kAddrWide, true, blocks_for(g.N, adjoint_block<ST>()));
+        ELBM_ADJOINT(kAddrWide, false, blocks_for(g.N, adjoint_block<ST>()));
     }
-    return cudaGetLastError();
+#define ELBM_ADJOINT_32(STT)                                                                           \
+    {                                                                                                  \
+        using ST = STT;                                                                                \
+        const dim3 planes(blocks_for(plane, adjoint_block<ST>()), unsigned(g.nz));                     \
+        const unsigned line = blocks_for(g.N, adjoint_block<ST>());                                    \
+        if (bytes && forced) ELBM_ADJOINT(kAddrBytes, true, planes);                                   \
+        if (bytes) ELBM_ADJOINT(kAddrBytes, false, planes);                                            \
+        if (forced) ELBM_ADJOINT(kAddrWide, true, line);                                               \
+        ELBM_ADJOINT(kAddrWide, false, line);                                                          \
+    }
+    switch (storage) {
+    case ELBM_STORE_F32: ELBM_ADJOINT_32(StoreF32)
+    case ELBM_STORE_F32DEV: ELBM_ADJOINT_32(StoreF32Dev)
+    case ELBM_STORE_F16DEV: ELBM_ADJOINT_32(StoreF16Dev)
+    case ELBM_STORE_BF16DEV: ELBM_ADJOINT_32(StoreBF16Dev)
+    default: return cudaErrorInvalidValue;
+    }
+#undef ELBM_ADJOINT_32
+#undef ELBM_ADJOINT
 }
 
 cudaError_t ELBM_CAT(launch_kinetic_energy, ELBM_SUFFIX)(int storage, const void *f, const Geometry &g, double rho0,
