@@ -997,11 +997,17 @@ __device__ __forceinline__ float2 node_collide_x2(float2 (&f)[9], float2 (&x)[9]
         }
         const float2 xi = pmul(delta, prcp(fval(i)));
         x[i] = xi;
-        xabs[0] = fmaxf(xabs[0], fabsf(xi.x));
-        xabs[1] = fmaxf(xabs[1], fabsf(xi.y));
-        xmin[0] = fminf(xmin[0], xi.x);
-        xmin[1] = fminf(xmin[1], xi.y);
+        if (i & 1) { // two populations at a time: three-input max and min
+            xabs[0] = fmaxf(xabs[0], fmaxf(fabsf(x[i - 1].x), fabsf(xi.x)));
+            xabs[1] = fmaxf(xabs[1], fmaxf(fabsf(x[i - 1].y), fabsf(xi.y)));
+            xmin[0] = fminf(xmin[0], fminf(x[i - 1].x, xi.x));
+            xmin[1] = fminf(xmin[1], fminf(x[i - 1].y, xi.y));
+        }
     }
+    xabs[0] = fmaxf(xabs[0], fabsf(x[Q - 1].x));
+    xabs[1] = fmaxf(xabs[1], fabsf(x[Q - 1].y));
+    xmin[0] = fminf(xmin[0], x[Q - 1].x);
+    xmin[1] = fminf(xmin[1], x[Q - 1].y);
 
     float2 alpha = f2(2.0f);
     br[0] = br[1] = kBranchCutoff;

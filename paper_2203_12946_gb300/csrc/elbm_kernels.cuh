@@ -139,6 +139,61 @@ __device__ __forceinline__ S *at(S *base, uint32_t o)
 }
 __device__ __forceinline__ uint32_t div_row(uint32_t n, RowDiv r) { return (__umulhi(r.magic, n) + n) >> r.shift; }
 
+// Two nodes x = xa and xa + 32 of row y of a D2Q9 domain (nx by ny, N nodes, populations at
+// in / out): pull, collide (node_collide_x2), store.  Where the warp's 64-node run lies inside
+// the row, clear of its ends, the second node's addresses are the first's plus 32 elements, an
+// immediate offset (32-bit byte offsets cost three integer instructions per address, 108 of
+// the 460 instructions of 64 nodes).  Else the columns wrap, and a second node past the end
+// of the row is a copy of the first, collided and not stored.  Plain loads when kCoherent
+// (buffers written during the launch), else ld_pop.
+template <class ST, int kAddr, bool kCoherent = false, bool kForce = false>
+__device__ __forceinline__ void step2_row(const typename ST::S *in, typename ST::S *out, uint32_t nx, uint32_t ny,
+                                          uint32_t N, uint32_t xa, uint32_t y, const CollideParams &p)
+{
+    using S = typename ST::S;
+    using T = typename ST::T;
+    constexpr uint32_t H = kPairSpan / 2;
+    constexpr uint32_t B = kAddr == kAddrBytes ? uint32_t(sizeof(S)) : 1u;
+    auto ld = [](const S *q) { return kCoherent ? *q : ld_pop<false>(q); };
+    const uint32_t sy[3] = {y == ny - 1 ? 0 : (y + 1) * nx, y * nx, (y == 0 ? ny - 1 : y - 1) * nx};
+    auto row = [&](int i) { return (uint32_t(i) * N + sy[vel(D, i, 1) + 1]) * B; };
+    const uint32_t run = xa & ~(H - 1); // first node of the warp's run (the same for the whole warp)
+    const bool inside = run >= 1 && run + kPairSpan < nx, hasb = xa + H < nx;
+    T fa[Q], fb[Q];
+    if (inside) {
+#pragma unroll
+        for (int i = 0; i < Q; ++i) {
+            const S *q = at<kAddr>(in, (xa - uint32_t(vel(D, i, 0))) * B + row(i));
+            fa[i] = ST::raw(ld(q));
+            fb[i] = ST::raw(ld(q + H));
+        }
+    } else {
+        const uint32_t xb = hasb ? xa + H : xa;
+        const uint32_t ca[3] = {xa == nx - 1 ? 0 : xa + 1, xa, xa == 0 ? nx - 1 : xa - 1};
+        const uint32_t cb[3] = {xb == nx - 1 ? 0 : xb + 1, xb, xb == 0 ? nx - 1 : xb - 1};
+#pragma unroll
+        for (int i = 0; i < Q; ++i) fa[i] = ST::raw(ld(at<kAddr>(in, ca[vel(D, i, 0) + 1] * B + row(i))));
+#pragma unroll
+        for (int i = 0; i < Q; ++i) fb[i] = ST::raw(ld(at<kAddr>(in, cb[vel(D, i, 0) + 1] * B + row(i))));
+    }
+    collide2_stored<D, ST, true>(fa, fb, p);
+    if constexpr (kForce) {
+        add_force<D, T, ST::kDev>(fa, p);
+        add_force<D, T, ST::kDev>(fb, p);
+    }
+    const uint32_t na = (y * nx + xa) * B;
+    auto st = [](S *q, S v) {
+        if (kCoherent) *q = v;
+        else __stcs(q, v);
+    };
+#pragma unroll
+    for (int i = 0; i < Q; ++i) {
+        S *q = at<kAddr>(out, uint32_t(i) * N * B + na);
+        st(q, ST::pack(fa[i]));
+        if (hasb) st(q + H, ST::pack(fb[i]));
+    }
+}
+
 template <class ST, int kAddr, bool kForce = false>
 __global__ void ELBM_STEP_BOUNDS k_step(const typename ST::S *__restrict__ fin,
                                                     typename ST::S *__restrict__ fout, Geometry g,
@@ -150,37 +205,13 @@ __global__ void ELBM_STEP_BOUNDS k_step(const typename ST::S *__restrict__ fin,
     if constexpr (nodes_per_thread<D, ST>() == 2) {
         // Two nodes per thread (pair_node); a second node past the end of the row (or of
         // the domain) is a copy of the first, collided and not stored.
-        constexpr uint32_t H = kPairSpan / 2;
-        T fa[Q], fb[Q];
         if constexpr (kAddr != kAddrWide) {
-            const uint32_t nx = uint32_t(g.nx), ny = uint32_t(g.ny), N = uint32_t(g.N);
             const uint32_t xa = blockIdx.x * kStepBlock + pair_node(threadIdx.x);
-            if (xa >= nx) return;
-            const bool hasb = xa + H < nx;
-            const uint32_t xb = hasb ? xa + H : xa;
-            const uint32_t y = blockIdx.y;
-            constexpr uint32_t B = kAddr == kAddrBytes ? uint32_t(sizeof(S)) : 1u;
-            const uint32_t ca[3] = {xa == nx - 1 ? 0 : xa + 1, xa, xa == 0 ? nx - 1 : xa - 1};
-            const uint32_t cb[3] = {xb == nx - 1 ? 0 : xb + 1, xb, xb == 0 ? nx - 1 : xb - 1};
-            const uint32_t sy[3] = {y == ny - 1 ? 0 : (y + 1) * nx, y * nx, (y == 0 ? ny - 1 : y - 1) * nx};
-            auto row = [&](int i) { return (uint32_t(i) * N + sy[vel(D, i, 1) + 1]) * B; };
-#pragma unroll
-            for (int i = 0; i < Q; ++i) fa[i] = ST::raw(ld_pop<false>(at<kAddr>(fin, ca[vel(D, i, 0) + 1] * B + row(i))));
-#pragma unroll
-            for (int i = 0; i < Q; ++i) fb[i] = ST::raw(ld_pop<false>(at<kAddr>(fin, cb[vel(D, i, 0) + 1] * B + row(i))));
-            collide2_stored<D, ST, true>(fa, fb, p);
-            if constexpr (kForce) {
-                add_force<D, T, ST::kDev>(fa, p);
-                add_force<D, T, ST::kDev>(fb, p);
-            }
-            const uint32_t na = (y * nx + xa) * B, nb = (y * nx + xb) * B;
-#pragma unroll
-            for (int i = 0; i < Q; ++i) __stcs(at<kAddr>(fout, uint32_t(i) * N * B + na), ST::pack(fa[i]));
-            if (hasb) {
-#pragma unroll
-                for (int i = 0; i < Q; ++i) __stcs(at<kAddr>(fout, uint32_t(i) * N * B + nb), ST::pack(fb[i]));
-            }
+            if (xa >= uint32_t(g.nx)) return;
+            step2_row<ST, kAddr, false, kForce>(fin, fout, uint32_t(g.nx), uint32_t(g.ny), uint32_t(g.N), xa, blockIdx.y, p);
         } else {
+            constexpr uint32_t H = kPairSpan / 2;
+            T fa[Q], fb[Q];
             const int64_t na = (int64_t)blockIdx.x * kStepBlock + pair_node(threadIdx.x);
             if (na >= g.N) return;
             const bool hasb = na + H < g.N;
@@ -953,49 +984,6 @@ __global__ void __launch_bounds__(kStepBlock, step_diag_min_blocks<ST>()) k_step
     diag_finish<kStepBlock>(dt, acc, s_hist);
 }
 
-// Two nodes x and x + 32 of row y of a D2Q9 domain (nx by ny, N nodes, populations
-// at in / out): pull, collide (node_collide_x2), store; a second node past the end of
-// the row is a copy of the first, collided and not stored.  Plain loads when kCoherent
-// (buffers written during the launch), else ld_pop.
-template <class ST, bool kCoherent = false>
-__device__ __forceinline__ void step2_row(const typename ST::S *in, typename ST::S *out, uint32_t nx, uint32_t ny,
-                                          uint32_t N, uint32_t xa, uint32_t y, const CollideParams &p)
-{
-    using T = typename ST::T;
-    constexpr uint32_t H = kPairSpan / 2;
-    const bool hasb = xa + H < nx;
-    const uint32_t xb = hasb ? xa + H : xa;
-    const uint32_t ym = y == 0 ? ny - 1 : y - 1, yp = y == ny - 1 ? 0 : y + 1;
-    auto src = [&](uint32_t x, int i) -> uint32_t {
-        const int cx = vel(D, i, 0), cy = vel(D, i, 1);
-        const uint32_t sx = cx == 1 ? (x == 0 ? nx - 1 : x - 1) : (cx == -1 ? (x == nx - 1 ? 0 : x + 1) : x);
-        const uint32_t sy = cy == 1 ? ym : (cy == -1 ? yp : y);
-        return uint32_t(i) * N + sy * nx + sx;
-    };
-    auto ld = [&](uint32_t o) { return kCoherent ? in[o] : ld_pop<false>(in + o); };
-    T fa[Q], fb[Q];
-#pragma unroll
-    for (int i = 0; i < Q; ++i) fa[i] = ST::raw(ld(src(xa, i)));
-#pragma unroll
-    for (int i = 0; i < Q; ++i) fb[i] = ST::raw(ld(src(xb, i)));
-    collide2_stored<D, ST, true>(fa, fb, p);
-    const uint32_t na = y * nx + xa, nb = y * nx + xb;
-#pragma unroll
-    for (int i = 0; i < Q; ++i) {
-        const typename ST::S v = ST::pack(fa[i]);
-        if (kCoherent) out[uint32_t(i) * N + na] = v;
-        else __stcs(out + (uint32_t(i) * N + na), v);
-    }
-    if (hasb) {
-#pragma unroll
-        for (int i = 0; i < Q; ++i) {
-            const typename ST::S v = ST::pack(fb[i]);
-            if (kCoherent) out[uint32_t(i) * N + nb] = v;
-            else __stcs(out + (uint32_t(i) * N + nb), v);
-        }
-    }
-}
-
 // --------------------------------------------------------------------------
 // --------------------------------------------------------------------------
 // Batched ensemble: one launch advances up to kBatchTableDomains domains.  Block
@@ -1049,7 +1037,7 @@ __global__ void __launch_bounds__(BX / nodes_per_thread<D, ST>(), batch_min_bloc
     typename ST::S *out = fout + dm.off;
     if constexpr (nodes_per_thread<D, ST>() == 2) {
         // two nodes per thread (D2Q9: z = 0), as in k_step
-        step2_row<ST>(in, out, nx, ny, N, x, y, p);
+        step2_row<ST, kAddrElems>(in, out, nx, ny, N, x, y, p);
         return;
     }
     const uint32_t xm = x == 0 ? nx - 1 : x - 1, xp = x == nx - 1 ? 0 : x + 1;
@@ -1153,7 +1141,7 @@ __global__ void __launch_bounds__(BX / nodes_per_thread<D, ST>()) k_step_persist
             }
             if (x >= nx) continue;
             if constexpr (nodes_per_thread<D, ST>() == 2) {
-                step2_row<ST, true>(in, out, nx, ny, N, x, yc, p);
+                step2_row<ST, kAddrElems, true>(in, out, nx, ny, N, x, yc, p);
                 continue;
             }
             const uint32_t y = yc, z = zc;
