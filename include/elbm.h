@@ -211,7 +211,9 @@ int elbm_set_stream(elbm_t *h, void *stream);
 int elbm_init_equilibrium(elbm_t *h, const double *rho, const double *u, int where);
 
 /* Advances the state by n >= 0 time steps (one fused pull-stream + collide
- * kernel launch per step, ping-pong between the two buffers).  Asynchronous.
+ * kernel launch per step, ping-pong between the two buffers; small D2Q9
+ * domains with FP32 arithmetic take up to four steps per launch under
+ * ELBM_KERNEL_AUTO, with the same result bit for bit).  Asynchronous.
  * Errors: ELBM_ERR_ARG (n < 0), ELBM_ERR_UNSUPPORTED (opts.kernel ==
  * ELBM_KERNEL_ROWS where it does not apply), ELBM_ERR_CUDA (launch failure).
  * A bounded device-side wait of the ROWS kernel that expires is reported as

@@ -404,12 +404,18 @@ int elbm_step(elbm_t *h, int64_t n)
     if (!h->pop[0]) return fail(h, ELBM_ERR_ARG, "elbm_step: no state (call elbm_init_equilibrium first)");
     DeviceGuard guard(h->opts.device);
     const CollideParams p = params_of(h);
-    for (int64_t k = 0; k < n; ++k) {
+    // n steps in as few launches as the kernel can take and of n's parity, so that the state
+    // ends in the buffer that one launch per step would leave it in; as even as they come
+    const int64_t most = ELBM_BY_LATTICE(h, steps_per_launch, h->opts.storage, h->g, h->opts.kernel, h->num_sms);
+    int64_t launches = (n + most - 1) / most;
+    launches += (launches ^ n) & 1;
+    for (int64_t k = 0; k < launches; ++k) {
+        const int steps = int(n / launches + (k < n % launches));
         cudaError_t e = ELBM_BY_LATTICE(h, launch_step, h->opts.storage, h->pop[h->cur], h->pop[h->cur ^ 1], h->g, p,
-                                        h->opts.kernel, h->num_sms, h->err_word, h->stream);
+                                        h->opts.kernel, steps, h->num_sms, h->err_word, h->stream);
         if (e != cudaSuccess) return cuda_fail(h, e, "elbm_step: kernel launch");
         h->cur ^= 1;
-        h->steps += 1;
+        h->steps += steps;
     }
     return ELBM_OK;
 }

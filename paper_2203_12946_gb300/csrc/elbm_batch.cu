@@ -509,9 +509,9 @@ int elbm_batch_step(elbm_batch_t *b, int64_t n, int mode)
                 const void *fin = static_cast<const char *>(b->pop[b->cur]) + size_t(dm.off) * b->elem;
                 void *fout = static_cast<char *>(b->pop[b->cur ^ 1]) + size_t(dm.off) * b->elem;
                 e = b->D == 2 ? eelbm::launch_step_d2q9(b->opts.storage, fin, fout, geom_of(dm), params_of(b, dm.beta),
-                                                        ELBM_KERNEL_DIRECT, b->num_sms, nullptr, b->stream)
+                                                        ELBM_KERNEL_DIRECT, 1, b->num_sms, nullptr, b->stream)
                               : eelbm::launch_step_d3q27(b->opts.storage, fin, fout, geom_of(dm),
-                                                         params_of(b, dm.beta), ELBM_KERNEL_DIRECT, b->num_sms,
+                                                         params_of(b, dm.beta), ELBM_KERNEL_DIRECT, 1, b->num_sms,
                                                          nullptr, b->stream);
                 if (e != cudaSuccess) return bcuda(b, e, "elbm_batch_step: per-domain launch");
             }

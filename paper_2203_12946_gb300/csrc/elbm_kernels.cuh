@@ -986,6 +986,84 @@ __global__ void __launch_bounds__(kStepBlock, step_diag_min_blocks<ST>()) k_step
 
 // --------------------------------------------------------------------------
 // --------------------------------------------------------------------------
+// Several steps of a small D2Q9 domain in one launch.  A step of a small domain costs its
+// latency, not its work: the launch, one pull from L2, one pass through the collision's chain
+// of dependent instructions (64^2: 1.7 us, of which the collision is 0.7).  Here a block
+// advances `rows` whole rows by k steps: it computes the first step of its rows and of the
+// k - 1 rows on either side from the input, each later step, one row fewer on either side,
+// from the one before in shared memory, and the last into the output.  The rows of the halos
+// are collided by more than one block, on SMs that would be idle.  A warp takes the same nodes
+// of a row as in step2_row and the state between two steps is rounded as it is stored, so the
+// result is that of k launches of k_step, bit for bit.  us per step, k_step and this kernel:
+// 64^2 1.71, 1.14; 64 x 256 2.33, 1.67; 100 x 90 1.89, 1.53; 128^2 2.56, 2.01.  Strips of
+// columns with halos of their own are no faster (64^2 1.05, 128^2 1.79) and would regroup the
+// nodes of a warp.
+constexpr int kTileThreads = 384;
+template <class ST, bool kForce = false>
+__global__ void __launch_bounds__(kTileThreads, 1) k_step_tile(const typename ST::S *__restrict__ fin,
+                                                              typename ST::S *__restrict__ fout, Geometry g,
+                                                              CollideParams p, int k, int rows)
+{
+    using S = typename ST::S;
+    using T = typename ST::T;
+    wait_previous_kernel();
+    extern __shared__ float s_tile[];
+    constexpr int H = int(kPairSpan) / 2;
+    const int nx = g.nx, ny = g.ny, R = rows + 2 * (k - 1);
+    const int y0 = int(blockIdx.x) * rows, h = min(rows, ny - y0);
+    // row r of the tile is row y0 - (k - 1) + r of the domain.  The odd steps write rows 0 .. R - 1
+    // of one buffer, the even ones, never the outermost rows, rows 1 .. R - 2 of the other
+    S *const odd = reinterpret_cast<S *>(s_tile), *const even = odd + Q * R * nx - nx;
+    const int runs = (nx + int(kPairSpan) - 1) / int(kPairSpan);
+    const int r0 = int(threadIdx.x >> 5) / runs, xa = (int(threadIdx.x >> 5) - r0 * runs) * int(kPairSpan) + int(threadIdx.x & 31);
+    const bool hasb = xa + H < nx;
+    const int xb = hasb ? xa + H : xa;
+    const int ca[3] = {xa == nx - 1 ? 0 : xa + 1, xa, xa == 0 ? nx - 1 : xa - 1};
+    const int cb[3] = {xb == nx - 1 ? 0 : xb + 1, xb, xb == 0 ? nx - 1 : xb - 1};
+    for (int step = 1; step <= k; ++step) {
+        const bool is_odd = step & 1;
+        const S *from = is_odd ? even : odd;
+        S *to = is_odd ? odd : even;
+        const int from_plane = (is_odd ? R - 2 : R) * nx, to_plane = (is_odd ? R : R - 2) * nx;
+        const int halo = k - step, row = r0 + step - 1; // one row of the step per warp run
+        if (r0 < h + 2 * halo && xa < nx) {
+            T fa[Q], fb[Q];
+            if (step == 1) {
+                int y = (y0 - halo + r0) % ny;
+                if (y < 0) y += ny;
+                const int sy[3] = {y == ny - 1 ? 0 : (y + 1) * nx, y * nx, (y == 0 ? ny - 1 : y - 1) * nx};
+#pragma unroll
+                for (int i = 0; i < Q; ++i) {
+                    const S *q = fin + (i * int(g.N) + sy[vel(D, i, 1) + 1]);
+                    fa[i] = ST::raw(ld_pop<false>(q + ca[vel(D, i, 0) + 1]));
+                    fb[i] = ST::raw(ld_pop<false>(q + cb[vel(D, i, 0) + 1]));
+                }
+            } else {
+#pragma unroll
+                for (int i = 0; i < Q; ++i) {
+                    const S *q = from + i * from_plane + (row - vel(D, i, 1)) * nx;
+                    fa[i] = ST::raw(q[ca[vel(D, i, 0) + 1]]);
+                    fb[i] = ST::raw(q[cb[vel(D, i, 0) + 1]]);
+                }
+            }
+            collide2_stored<D, ST, true>(fa, fb, p);
+            if constexpr (kForce) {
+                add_force<D, T, ST::kDev>(fa, p);
+                add_force<D, T, ST::kDev>(fb, p);
+            }
+            S *q = step < k ? to + row * nx + xa : fout + ((y0 + r0) * nx + xa);
+            const int plane = step < k ? to_plane : int(g.N);
+#pragma unroll
+            for (int i = 0; i < Q; ++i, q += plane) {
+                q[0] = ST::pack(fa[i]);
+                if (hasb) q[H] = ST::pack(fb[i]);
+            }
+        }
+        if (step < k) __syncthreads();
+    }
+}
+
+// --------------------------------------------------------------------------
 // Batched ensemble: one launch advances up to kBatchTableDomains domains.  Block
 // b is one work item, nodes x0 .. x0 + BX - 1 of one x-row of one domain; the
 // block finds its domain in the launch's parameter table (a coarse index, then a
@@ -1431,7 +1509,7 @@ static inline unsigned blocks_for(int64_t N, int block) { return unsigned((N + b
 
 // Launches a kernel that begins with wait_previous_kernel().
 template <class... P, class... A>
-cudaError_t launch(void (*kernel)(P...), dim3 grid, unsigned block, cudaStream_t s, A &&...args)
+cudaError_t launch_shared(void (*kernel)(P...), dim3 grid, unsigned block, size_t shared, cudaStream_t s, A &&...args)
 {
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute attr[1];
@@ -1439,12 +1517,18 @@ cudaError_t launch(void (*kernel)(P...), dim3 grid, unsigned block, cudaStream_t
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.gridDim = grid;
     cfg.blockDim = dim3(block);
+    cfg.dynamicSmemBytes = shared;
     cfg.stream = s;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
     if (e != cudaSuccess) cudaGetLastError(); // reported here, not by the caller's next CUDA call
     return e;
+}
+template <class... P, class... A>
+cudaError_t launch(void (*kernel)(P...), dim3 grid, unsigned block, cudaStream_t s, A &&...args)
+{
+    return launch_shared(kernel, grid, block, 0, s, static_cast<A &&>(args)...);
 }
 
 } // namespace ELBM_SUFFIX
@@ -1516,9 +1600,24 @@ bool ELBM_CAT(rows_kernel_applies, ELBM_SUFFIX)(int storage, const Geometry &g)
     }
 }
 
+// Most steps that one launch_step takes with this kernel choice (1 but for k_step_tile).
+// k_step_tile is for domains whose work one wave of blocks of two rows can take several times:
+// rows of at most two warps and no more row pairs than SMs.  Rows of more warps lose the
+// latency again to the halo's work (203 x 177: 2.95 us per step by k_step, 2.89 so; 203 x 100
+// 2.64, 2.85).  Four steps for rows of one warp, three for two (128^2: 2.01 us per step
+// against 2.07 with four, and within 48 KB of shared memory).
+constexpr int kTileRows = 2;
+int ELBM_CAT(steps_per_launch, ELBM_SUFFIX)(int storage, const Geometry &g, int kernel, int num_sms)
+{
+    using namespace ELBM_SUFFIX;
+    if (D != 2 || storage == ELBM_STORE_F64 || kernel != ELBM_KERNEL_AUTO) return 1;
+    if (g.N == 0 || g.nx > 2 * int(kPairSpan) || (g.ny + kTileRows - 1) / kTileRows > num_sms) return 1;
+    return g.nx <= int(kPairSpan) ? 4 : 3;
+}
+
 cudaError_t ELBM_CAT(launch_step, ELBM_SUFFIX)(int storage, const void *fin, void *fout,
                                                const Geometry &g, const CollideParams &p, int kernel,
-                                               int num_sms, int *err, cudaStream_t s)
+                                               int steps, int num_sms, int *err, cudaStream_t s)
 {
     using namespace ELBM_SUFFIX;
     if (g.N == 0) return cudaSuccess;
@@ -1547,6 +1646,30 @@ cudaError_t ELBM_CAT(launch_step, ELBM_SUFFIX)(int storage, const void *fin, voi
 #undef ELBM_ROWS_FOR
     }
     if (kernel == ELBM_KERNEL_ROWS) return cudaErrorNotSupported;
+    if (steps > 1) {
+        if (steps > ELBM_CAT(steps_per_launch, ELBM_SUFFIX)(storage, g, kernel, num_sms)) return cudaErrorInvalidValue;
+        if constexpr (D == 2) {
+            const unsigned R = unsigned(kTileRows + 2 * (steps - 1)), nx = unsigned(g.nx);
+            const unsigned threads = R * ((nx + kPairSpan - 1) / kPairSpan) * 32u; // at most kTileThreads
+            const size_t shared = size_t(Q) * (R + R - 2) * nx * (storage == ELBM_STORE_F32 || storage == ELBM_STORE_F32DEV ? 4 : 2);
+            const unsigned grid = unsigned((g.ny + kTileRows - 1) / kTileRows);
+#define ELBM_TILE(FORCE)                                                                                    \
+    switch (storage) {                                                                                      \
+    case ELBM_STORE_F32: { using ST = StoreF32; ELBM_TILE_ONE(FORCE); }                                     \
+    case ELBM_STORE_F32DEV: { using ST = StoreF32Dev; ELBM_TILE_ONE(FORCE); }                               \
+    case ELBM_STORE_F16DEV: { using ST = StoreF16Dev; ELBM_TILE_ONE(FORCE); }                               \
+    default: { using ST = StoreBF16Dev; ELBM_TILE_ONE(FORCE); }                                             \
+    }
+#define ELBM_TILE_ONE(FORCE)                                                                                \
+    return launch_shared(k_step_tile<ST, FORCE>, grid, threads, shared, s,                                  \
+                         static_cast<const typename ST::S *>(fin), static_cast<typename ST::S *>(fout), g,  \
+                         p, steps, kTileRows)
+            if (forced) ELBM_TILE(true)
+            ELBM_TILE(false)
+#undef ELBM_TILE
+#undef ELBM_TILE_ONE
+        }
+    }
     const uint64_t elems = uint64_t(Q) * uint64_t(g.N);
     const RowDiv rd = row_div(uint32_t(g.nx));
 #define ELBM_DIRECT_STEP(ADDR, GRID)                                                                   \
