@@ -619,9 +619,9 @@ int elbm_get_populations(elbm_t *h, void *dst, int where)
         return fail(h, ELBM_ERR_ARG, "elbm_get_populations: bad memory location %d", where);
     if (!h->pop[0]) return fail(h, ELBM_ERR_ARG, "elbm_get_populations: no state");
     DeviceGuard guard(h->opts.device);
-    cudaError_t e = cudaMemcpyAsync(dst, h->pop[h->cur], h->pop_bytes,
-                                    where == ELBM_MEM_HOST ? cudaMemcpyDeviceToHost : cudaMemcpyDeviceToDevice,
-                                    h->stream);
+    cudaError_t e = where == ELBM_MEM_HOST
+                        ? cudaMemcpyAsync(dst, h->pop[h->cur], h->pop_bytes, cudaMemcpyDeviceToHost, h->stream)
+                        : eelbm::copy_device(dst, h->pop[h->cur], dst, h->pop_bytes, h->opts.device, h->stream);
     if (e == cudaSuccess && where == ELBM_MEM_HOST) e = cudaStreamSynchronize(h->stream);
     if (e != cudaSuccess) return cuda_fail(h, e, "elbm_get_populations");
     if (where == ELBM_MEM_HOST) return check_device_flag(h, "elbm_get_populations");
@@ -637,9 +637,9 @@ int elbm_set_populations(elbm_t *h, const void *src, int where)
     DeviceGuard guard(h->opts.device);
     int st = ensure_populations(h);
     if (st != ELBM_OK) return st;
-    cudaError_t e = cudaMemcpyAsync(h->pop[0], src, h->pop_bytes,
-                                    where == ELBM_MEM_HOST ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToDevice,
-                                    h->stream);
+    cudaError_t e = where == ELBM_MEM_HOST
+                        ? cudaMemcpyAsync(h->pop[0], src, h->pop_bytes, cudaMemcpyHostToDevice, h->stream)
+                        : eelbm::copy_device(h->pop[0], src, src, h->pop_bytes, h->opts.device, h->stream);
     if (e == cudaSuccess && where == ELBM_MEM_HOST) e = cudaStreamSynchronize(h->stream);
     if (e != cudaSuccess) return cuda_fail(h, e, "elbm_set_populations");
     h->cur = 0;

@@ -792,9 +792,10 @@ int elbm_batch_get_populations(elbm_batch_t *b, int domain, void *dst, int where
     DeviceGuard guard(b->opts.device);
     const BatchDomain &dm = b->doms[domain];
     const void *src = static_cast<const char *>(b->pop[b->cur]) + size_t(dm.off) * b->elem;
-    cudaError_t e = cudaMemcpyAsync(dst, src, size_t(b->Q) * size_t(dm.N) * b->elem,
-                                    where == ELBM_MEM_HOST ? cudaMemcpyDeviceToHost : cudaMemcpyDeviceToDevice,
-                                    b->stream);
+    const size_t bytes = size_t(b->Q) * size_t(dm.N) * b->elem;
+    cudaError_t e = where == ELBM_MEM_HOST
+                        ? cudaMemcpyAsync(dst, src, bytes, cudaMemcpyDeviceToHost, b->stream)
+                        : eelbm::copy_device(dst, src, dst, bytes, b->opts.device, b->stream);
     if (e == cudaSuccess && where == ELBM_MEM_HOST) e = cudaStreamSynchronize(b->stream);
     if (e != cudaSuccess) return bcuda(b, e, "elbm_batch_get_populations");
     return ELBM_OK;
@@ -811,9 +812,11 @@ int elbm_batch_set_populations(elbm_batch_t *b, int domain, const void *src, int
     const size_t bytes = size_t(b->Q) * size_t(dm.N) * b->elem;
     cudaError_t e = cudaSuccess;
     // write both buffers so that the step parity does not matter
-    for (int k = 0; k < 2 && e == cudaSuccess; ++k)
-        e = cudaMemcpyAsync(static_cast<char *>(b->pop[k]) + size_t(dm.off) * b->elem, src, bytes,
-                            where == ELBM_MEM_HOST ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToDevice, b->stream);
+    for (int k = 0; k < 2 && e == cudaSuccess; ++k) {
+        void *dst = static_cast<char *>(b->pop[k]) + size_t(dm.off) * b->elem;
+        e = where == ELBM_MEM_HOST ? cudaMemcpyAsync(dst, src, bytes, cudaMemcpyHostToDevice, b->stream)
+                                   : eelbm::copy_device(dst, src, src, bytes, b->opts.device, b->stream);
+    }
     if (e == cudaSuccess && where == ELBM_MEM_HOST) e = cudaStreamSynchronize(b->stream);
     if (e != cudaSuccess) return bcuda(b, e, "elbm_batch_set_populations");
     return ELBM_OK;

@@ -1507,30 +1507,6 @@ __global__ void __launch_bounds__(kAuxBlock) k_equilibrium_vjp(const double *__r
 
 static inline unsigned blocks_for(int64_t N, int block) { return unsigned((N + block - 1) / block); }
 
-// Launches a kernel that begins with wait_previous_kernel().
-template <class... P, class... A>
-cudaError_t launch_shared(void (*kernel)(P...), dim3 grid, unsigned block, size_t shared, cudaStream_t s, A &&...args)
-{
-    cudaLaunchConfig_t cfg = {};
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.gridDim = grid;
-    cfg.blockDim = dim3(block);
-    cfg.dynamicSmemBytes = shared;
-    cfg.stream = s;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
-    if (e != cudaSuccess) cudaGetLastError(); // reported here, not by the caller's next CUDA call
-    return e;
-}
-template <class... P, class... A>
-cudaError_t launch(void (*kernel)(P...), dim3 grid, unsigned block, cudaStream_t s, A &&...args)
-{
-    return launch_shared(kernel, grid, block, 0, s, static_cast<A &&>(args)...);
-}
-
 } // namespace ELBM_SUFFIX
 
 #define ELBM_CAT2(a, b) a##_##b

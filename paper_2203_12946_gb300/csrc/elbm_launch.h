@@ -90,6 +90,34 @@ __host__ __device__ inline double from_ordered_bits(unsigned long long o)
     return d;
 }
 
+// Launches a kernel that begins with wait_previous_kernel().
+template <class... P, class... A>
+cudaError_t launch_shared(void (*kernel)(P...), dim3 grid, unsigned block, size_t shared, cudaStream_t s, A &&...args)
+{
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(block);
+    cfg.dynamicSmemBytes = shared;
+    cfg.stream = s;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+    if (e != cudaSuccess) cudaGetLastError(); // reported here, not by the caller's next CUDA call
+    return e;
+}
+template <class... P, class... A>
+cudaError_t launch(void (*kernel)(P...), dim3 grid, unsigned block, cudaStream_t s, A &&...args)
+{
+    return launch_shared(kernel, grid, block, 0, s, static_cast<A &&>(args)...);
+}
+
+// dst <- src on stream s of the current device `device`; `outer`, one of the two, is the
+// caller's pointer, about which nothing is known (elbm_copy.cu).
+cudaError_t copy_device(void *dst, const void *src, const void *outer, size_t bytes, int device, cudaStream_t s);
+
 #define ELBM_DECLARE_LAUNCHERS(SUFFIX)                                                               \
     cudaError_t launch_step_##SUFFIX(int storage, const void *fin, void *fout, const Geometry &g,   \
                                      const CollideParams &p, int kernel, int steps, int num_sms,     \

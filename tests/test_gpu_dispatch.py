@@ -198,3 +198,47 @@ def test_kernels_of_a_stream_see_each_other_and_the_callers(D, dims, storage):
     want = go(True, None)
     assert torch.equal(go(False, None), want)
     assert torch.equal(go(False, torch.cuda.Stream()), want)
+
+
+@pytest.mark.parametrize("where", ["plain", "captured"])
+@pytest.mark.parametrize("offset", [0, 16, 8, 1])
+@pytest.mark.parametrize("D,dims,storage", [(2, (1, 1, 1), "f16dev"), (2, (7, 1, 1), "f32"), (2, (227, 1, 1), "f32"),
+                                            (2, (3641, 1, 1), "f16dev"), (3, (41, 13, 9), "f64")])
+def test_device_copies_of_populations(D, dims, storage, offset, where):
+    """Copies between device buffers, by the library's kernel where both ends lie on 16 bytes and
+    by the driver elsewhere: sizes with and without bytes left over, around one block's 8 KB,
+    nothing written beside them; also under capture."""
+    torch = pytest.importorskip("torch")
+    raw = raw_state(D, dims, storage)
+    with E.Simulation(LAT[D], dims, 0.97, storage=storage) as sim, \
+            E.Ensemble(LAT[D], [dims, dims], [0.9, 0.9], storage=storage) as ens:
+        n = sim.pop_bytes
+        out = torch.full((n + 64,), 0xA5, dtype=torch.uint8, device="cuda")
+        dst = out[offset:offset + n]
+        sim.set_populations(raw)
+        if where == "captured":
+            E.elbm_get_populations(sim.h, dst, E.ELBM_MEM_DEVICE)  # a first call outside
+            out.fill_(0xA5)
+            torch.cuda.synchronize()
+            graph, side = torch.cuda.CUDAGraph(), torch.cuda.Stream()
+            E.elbm_set_stream(sim.h, side.cuda_stream)
+            with torch.cuda.graph(graph, stream=side):
+                E.elbm_get_populations(sim.h, dst, E.ELBM_MEM_DEVICE)
+            graph.replay()
+        else:
+            E.elbm_get_populations(sim.h, dst, E.ELBM_MEM_DEVICE)
+        torch.cuda.synchronize()
+        want = np.full(n + 64, 0xA5, np.uint8)
+        want[offset:offset + n] = np.ascontiguousarray(raw).view(np.uint8).ravel()
+        assert np.array_equal(out.cpu().numpy(), want)
+        if where == "captured":
+            return
+        sim.set_populations(np.zeros_like(raw))
+        E.elbm_set_populations(sim.h, dst, E.ELBM_MEM_DEVICE)
+        E.elbm_batch_set_populations(ens.b, 1, dst, E.ELBM_MEM_DEVICE)
+        assert np.array_equal(sim.get_populations(), raw)
+        assert np.array_equal(ens.get_populations(1), raw)
+        out.fill_(0xA5)
+        E.elbm_batch_get_populations(ens.b, 1, dst, E.ELBM_MEM_DEVICE)
+        torch.cuda.synchronize()
+        assert np.array_equal(out.cpu().numpy(), want)
