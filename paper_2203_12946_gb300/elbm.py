@@ -105,6 +105,8 @@ def library_path() -> str:
 def load(build_if_missing: bool = True):
     """Load libelbm.so (building it first if it is missing and nvcc exists)."""
     global _lib
+    if _lib is not None:  # every call comes through here: no lock once it is set
+        return _lib
     with _lock:
         if _lib is not None:
             return _lib
@@ -175,16 +177,17 @@ def _ptr(x):
     """Address of a numpy array, torch tensor, ctypes object or integer (None -> NULL)."""
     if x is None:
         return None
+    data_ptr = getattr(x, "data_ptr", None)  # tensors first, the common case
+    if data_ptr is not None:
+        if not x.is_contiguous():
+            raise ValueError("tensor must be contiguous")
+        return data_ptr()
     if isinstance(x, int):
         return x
     if isinstance(x, np.ndarray):
         if not x.flags["C_CONTIGUOUS"]:
             raise ValueError("array must be C-contiguous")
         return x.ctypes.data
-    if hasattr(x, "data_ptr"):
-        if not x.is_contiguous():
-            raise ValueError("tensor must be contiguous")
-        return x.data_ptr()
     return ctypes.addressof(x)
 
 
@@ -480,7 +483,7 @@ class Simulation:
 
     def state_copy(self):
         """Device copy of the current populations (raw storage bytes)."""
-        buf = self.torch.empty(self.pop_bytes, dtype=self.torch.uint8, device=self.device)
+        buf = self.torch.empty_like(self.buffers[0])
         elbm_get_populations(self.h, buf, ELBM_MEM_DEVICE)
         return buf
 
