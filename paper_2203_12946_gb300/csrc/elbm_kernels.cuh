@@ -13,6 +13,7 @@
 //              then shared memory, then one atomic per block and quantity
 #pragma once
 
+#include <algorithm>
 #include <type_traits>
 
 #include "elbm_device.cuh"
@@ -194,6 +195,35 @@ __device__ __forceinline__ void step2_row(const typename ST::S *in, typename ST:
     }
 }
 
+// Node (x, y, z) of a domain: pull, collide, store.  The offsets of the nine (c_x, c_y) sources
+// in a plane are the thread's; the rest of an address is the same for the whole block.
+template <class ST, int kAddr, bool kForce = false>
+__device__ __forceinline__ void step1_node(const typename ST::S *in, typename ST::S *out, uint32_t nx, uint32_t ny,
+                                           uint32_t nz, uint32_t N, uint32_t x, uint32_t y, uint32_t z, const CollideParams &p)
+{
+    using S = typename ST::S;
+    using T = typename ST::T;
+    T f[Q], xd[Q]; // the stored values (deviations for deviation storage)
+    int br;
+    const uint32_t plane = nx * ny;
+    constexpr uint32_t B = kAddr == kAddrBytes ? uint32_t(sizeof(S)) : 1u;
+    const uint32_t sx[3] = {x == nx - 1 ? 0 : x + 1, x, x == 0 ? nx - 1 : x - 1};
+    const uint32_t sy[3] = {y == ny - 1 ? 0 : (y + 1) * nx, y * nx, (y == 0 ? ny - 1 : y - 1) * nx};
+    const uint32_t sz[3] = {z == nz - 1 ? 0 : z + 1, z, z == 0 ? nz - 1 : z - 1};
+#pragma unroll
+    for (int i = 0; i < Q; ++i) {
+        const int cx = vel(D, i, 0), cy = vel(D, i, 1), cz = D == 3 ? vel(D, i, 2) : 0;
+        const uint32_t o = (sy[cy + 1] + sx[cx + 1]) * B;
+        const uint32_t b = (uint32_t(i) * N + sz[cz + 1] * plane) * B;
+        f[i] = ST::raw(ld_pop<D == 3>(at<kAddr>(in, o + b)));
+    }
+    collide_stored<D, ST, true>(f, xd, p, &br);
+    if constexpr (kForce) add_force<D, T, ST::kDev>(f, p);
+    const uint32_t n = (z * plane + y * nx + x) * B;
+#pragma unroll
+    for (int i = 0; i < Q; ++i) __stcs(at<kAddr>(out, uint32_t(i) * N * B + n), ST::pack(f[i]));
+}
+
 template <class ST, int kAddr, bool kForce = false>
 __global__ void ELBM_STEP_BOUNDS k_step(const typename ST::S *__restrict__ fin,
                                                     typename ST::S *__restrict__ fout, Geometry g,
@@ -236,32 +266,15 @@ __global__ void ELBM_STEP_BOUNDS k_step(const typename ST::S *__restrict__ fin,
         }
         return;
     }
-    T f[Q], xd[Q]; // the stored values (deviations for deviation storage)
-    int br;
     if constexpr (kAddr != kAddrWide) {
         const uint32_t nx = uint32_t(g.nx), ny = uint32_t(g.ny), nz = uint32_t(g.nz), N = uint32_t(g.N);
         const uint32_t plane = nx * ny, xy = blockIdx.x * blockDim.x + threadIdx.x, z = blockIdx.y;
         if (xy >= plane) return;
         const uint32_t y = div_row(xy, rd), x = xy - y * nx;
-        // offsets of the nine (c_x, c_y) sources in a plane; the rest of an address is the
-        // same for the whole block
-        constexpr uint32_t B = kAddr == kAddrBytes ? uint32_t(sizeof(S)) : 1u;
-        const uint32_t sx[3] = {x == nx - 1 ? 0 : x + 1, x, x == 0 ? nx - 1 : x - 1};
-        const uint32_t sy[3] = {y == ny - 1 ? 0 : (y + 1) * nx, y * nx, (y == 0 ? ny - 1 : y - 1) * nx};
-        const uint32_t sz[3] = {z == nz - 1 ? 0 : z + 1, z, z == 0 ? nz - 1 : z - 1};
-#pragma unroll
-        for (int i = 0; i < Q; ++i) {
-            const int cx = vel(D, i, 0), cy = vel(D, i, 1), cz = D == 3 ? vel(D, i, 2) : 0;
-            const uint32_t o = (sy[cy + 1] + sx[cx + 1]) * B;
-            const uint32_t b = (uint32_t(i) * N + sz[cz + 1] * plane) * B;
-            f[i] = ST::raw(ld_pop<D == 3>(at<kAddr>(fin, o + b)));
-        }
-        collide_stored<D, ST, true>(f, xd, p, &br);
-        if constexpr (kForce) add_force<D, T, ST::kDev>(f, p);
-        const uint32_t n = (z * plane + xy) * B;
-#pragma unroll
-        for (int i = 0; i < Q; ++i) __stcs(at<kAddr>(fout, uint32_t(i) * N * B + n), ST::pack(f[i]));
+        step1_node<ST, kAddr, kForce>(fin, fout, nx, ny, nz, N, x, y, z, p);
     } else {
+        T f[Q], xd[Q]; // the stored values (deviations for deviation storage)
+        int br;
         const int64_t n = (int64_t)blockIdx.x * kStepBlock + threadIdx.x;
         if (n >= g.N) return;
         int x, y, z;
@@ -1068,9 +1081,11 @@ __global__ void __launch_bounds__(kTileThreads, 1) k_step_tile(const typename ST
 // b is one work item, nodes x0 .. x0 + BX - 1 of one x-row of one domain; the
 // block finds its domain in the launch's parameter table (a coarse index, then a
 // forward scan over the item counts) and its row by division, both uniform over the
-// block, so each thread then addresses its populations as k_step does (32-bit
-// offsets inside the domain).  Each domain has its own beta; everything else is the
-// single-domain step.
+// block, so each thread then addresses its populations as k_step does: 32-bit offsets
+// inside the domain, in bytes where every domain of the launch holds less than 2^32 bytes
+// (us per step, element offsets and bytes: 64 D2Q9 domains of 3.93 M nodes FP32 52.5, 51.8,
+// 16-bit 55.3, 54.1; 20 D3Q27 domains of 1.41 M nodes 73.4, 71.9 and 75.9, 71.5).  Each domain
+// has its own beta; everything else is the single-domain step.
 // --------------------------------------------------------------------------
 // Resident threads per SM requested from the register allocator for the batched ensemble
 // kernel (0: no bound).  Two-node D2Q9 kernels: 1024 (at most 64 registers; 74.7 against
@@ -1092,7 +1107,7 @@ constexpr int batch_min_blocks()
 {
     return batch_threads_per_sm<ST>() / (BX / nodes_per_thread<D, ST>());
 }
-template <class ST, int BX>
+template <class ST, int BX, int kAddr>
 __global__ void __launch_bounds__(BX / nodes_per_thread<D, ST>(), batch_min_blocks<ST, BX>()) k_step_batch(const typename ST::S *__restrict__ fin,
                                                   typename ST::S *__restrict__ fout,
                                                   const __grid_constant__ BatchTable tab, CollideParams p)
@@ -1115,27 +1130,10 @@ __global__ void __launch_bounds__(BX / nodes_per_thread<D, ST>(), batch_min_bloc
     typename ST::S *out = fout + dm.off;
     if constexpr (nodes_per_thread<D, ST>() == 2) {
         // two nodes per thread (D2Q9: z = 0), as in k_step
-        step2_row<ST, kAddrElems>(in, out, nx, ny, N, x, y, p);
+        step2_row<ST, kAddr>(in, out, nx, ny, N, x, y, p);
         return;
     }
-    const uint32_t xm = x == 0 ? nx - 1 : x - 1, xp = x == nx - 1 ? 0 : x + 1;
-    const uint32_t ym = y == 0 ? ny - 1 : y - 1, yp = y == ny - 1 ? 0 : y + 1;
-    const uint32_t zm = z == 0 ? nz - 1 : z - 1, zp = z == nz - 1 ? 0 : z + 1;
-    T f[Q], xd[Q];
-    auto src = [&](int i) -> uint32_t {
-        const int cx = vel(D, i, 0), cy = vel(D, i, 1), cz = D == 3 ? vel(D, i, 2) : 0;
-        const uint32_t sx = cx == 1 ? xm : (cx == -1 ? xp : x);
-        const uint32_t sy = cy == 1 ? ym : (cy == -1 ? yp : y);
-        const uint32_t sz = cz == 1 ? zm : (cz == -1 ? zp : z);
-        return uint32_t(i) * N + (sz * ny + sy) * nx + sx;
-    };
-#pragma unroll
-    for (int i = 0; i < Q; ++i) f[i] = ST::raw(ld_pop<false>(in + src(i)));
-    int br;
-    collide_stored<D, ST, true>(f, xd, p, &br);
-    const uint32_t n = (z * ny + y) * nx + x;
-#pragma unroll
-    for (int i = 0; i < Q; ++i) __stcs(out + (uint32_t(i) * N + n), ST::pack(f[i]));
+    step1_node<ST, kAddr>(in, out, nx, ny, nz, N, x, y, z, p);
 }
 
 // --------------------------------------------------------------------------
@@ -1505,6 +1503,10 @@ __global__ void __launch_bounds__(kAuxBlock) k_equilibrium_vjp(const double *__r
     default: return cudaErrorInvalidValue;                                                     \
     }
 
+static inline uint64_t storage_bytes(int storage)
+{
+    return storage == ELBM_STORE_F64 ? 8 : storage == ELBM_STORE_F32 || storage == ELBM_STORE_F32DEV ? 4 : 2;
+}
 static inline unsigned blocks_for(int64_t N, int block) { return unsigned((N + block - 1) / block); }
 
 } // namespace ELBM_SUFFIX
@@ -1512,8 +1514,9 @@ static inline unsigned blocks_for(int64_t N, int block) { return unsigned((N + b
 #define ELBM_CAT2(a, b) a##_##b
 #define ELBM_CAT(a, b) ELBM_CAT2(a, b)
 
-// A lattice may be compiled in two units: ELBM_PART 1 holds the step launcher (and the
-// row pipeline), ELBM_PART 2 every other launcher; without ELBM_PART one unit holds all.
+// A lattice may be compiled in three units: ELBM_PART 1 holds the step launcher (and the
+// row pipeline), ELBM_PART 3 the launchers of the batched ensemble, ELBM_PART 2 every other
+// launcher; without ELBM_PART one unit holds all.
 #if !defined(ELBM_PART) || ELBM_PART == 1
 namespace ELBM_SUFFIX {
 
@@ -1627,7 +1630,7 @@ cudaError_t ELBM_CAT(launch_step, ELBM_SUFFIX)(int storage, const void *fin, voi
         if constexpr (D == 2) {
             const unsigned R = unsigned(kTileRows + 2 * (steps - 1)), nx = unsigned(g.nx);
             const unsigned threads = R * ((nx + kPairSpan - 1) / kPairSpan) * 32u; // at most kTileThreads
-            const size_t shared = size_t(Q) * (R + R - 2) * nx * (storage == ELBM_STORE_F32 || storage == ELBM_STORE_F32DEV ? 4 : 2);
+            const size_t shared = size_t(Q) * (R + R - 2) * nx * storage_bytes(storage);
             const unsigned grid = unsigned((g.ny + kTileRows - 1) / kTileRows);
 #define ELBM_TILE(FORCE)                                                                                    \
     switch (storage) {                                                                                      \
@@ -1673,10 +1676,7 @@ cudaError_t ELBM_CAT(launch_step, ELBM_SUFFIX)(int storage, const void *fin, voi
             while (threads > 32 && int64_t(blocks_for(plane, threads)) * g.nz < 2 * int64_t(num_sms)) threads /= 2;
         const dim3 grid = pair ? dim3(blocks_for(g.nx, kStepBlock), unsigned(g.ny))
                                : dim3(blocks_for(plane, threads), unsigned(g.nz));
-        const uint64_t size = storage == ELBM_STORE_F64                                       ? 8
-                              : storage == ELBM_STORE_F32 || storage == ELBM_STORE_F32DEV ? 4
-                                                                                              : 2;
-        if (elems * size <= 0xffffffffull) {
+        if (elems * storage_bytes(storage) <= 0xffffffffull) {
             ELBM_DIRECT_STEP(kAddrBytes, grid)
         } else {
             ELBM_DIRECT_STEP(kAddrElems, grid)
@@ -1706,6 +1706,9 @@ cudaError_t ELBM_CAT(launch_step_diag, ELBM_SUFFIX)(int storage, const void *fin
     return cudaGetLastError();
 }
 
+#endif
+
+#if !defined(ELBM_PART) || ELBM_PART == 3
 cudaError_t ELBM_CAT(launch_step_batch, ELBM_SUFFIX)(int storage, const void *fin, void *fout,
                                                      const BatchTable &tab, int bx, const CollideParams &p,
                                                      cudaStream_t s)
@@ -1713,18 +1716,27 @@ cudaError_t ELBM_CAT(launch_step_batch, ELBM_SUFFIX)(int storage, const void *fi
     using namespace ELBM_SUFFIX;
     const int nitems = tab.item0[tab.n];
     if (tab.n <= 0 || nitems <= 0) return cudaSuccess;
-#define ELBM_BATCH_BX(BXV)                                                                             \
-    ELBM_STORAGE_SWITCH(storage, return launch(k_step_batch<ST, BXV>, unsigned(nitems), BXV / nodes_per_thread<D, ST>(), s, \
+    int64_t most = 0; // nodes of the largest domain
+    for (int d = 0; d < tab.n; ++d) most = std::max(most, int64_t(tab.dom[d].nx) * tab.dom[d].ny * tab.dom[d].nz);
+    const bool bytes = uint64_t(Q) * uint64_t(most) * storage_bytes(storage) <= 0xffffffffull;
+#define ELBM_BATCH_BX(BXV, ADDR)                                                                       \
+    ELBM_STORAGE_SWITCH(storage, return launch(k_step_batch<ST, BXV, ADDR>, unsigned(nitems), BXV / nodes_per_thread<D, ST>(), s, \
                                                static_cast<const typename ST::S *>(fin),               \
                                                static_cast<typename ST::S *>(fout), tab, p))
-    switch (bx) {
-    case 64: ELBM_BATCH_BX(64); break;
-    case 128: ELBM_BATCH_BX(128); break;
-    case 256: ELBM_BATCH_BX(256); break;
-    default: return cudaErrorInvalidValue;
+#define ELBM_BATCH_ADDR(ADDR)                                                                          \
+    switch (bx) {                                                                                      \
+    case 64: ELBM_BATCH_BX(64, ADDR); break;                                                           \
+    case 128: ELBM_BATCH_BX(128, ADDR); break;                                                         \
+    case 256: ELBM_BATCH_BX(256, ADDR); break;                                                         \
     }
+    if (bytes) {
+        ELBM_BATCH_ADDR(kAddrBytes)
+    } else {
+        ELBM_BATCH_ADDR(kAddrElems)
+    }
+    return cudaErrorInvalidValue; // bx
+#undef ELBM_BATCH_ADDR
 #undef ELBM_BATCH_BX
-    return cudaGetLastError();
 }
 
 cudaError_t ELBM_CAT(persist_blocks_per_sm, ELBM_SUFFIX)(int storage, int bx, int *blocks)
@@ -1775,6 +1787,9 @@ cudaError_t ELBM_CAT(launch_step_persist, ELBM_SUFFIX)(int storage, void *pop0, 
     return cudaErrorInvalidValue;
 }
 
+#endif
+
+#if !defined(ELBM_PART) || ELBM_PART == 2
 cudaError_t ELBM_CAT(launch_step_adjoint, ELBM_SUFFIX)(int storage, const void *fin, const void *gnext,
                                                        void *gout, const Geometry &g, const CollideParams &p,
                                                        double *dforce, cudaStream_t s)

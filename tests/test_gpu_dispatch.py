@@ -95,10 +95,20 @@ def test_populations_beyond_4_gb(D, small, tiles):
     with E.Simulation(LAT[D], big, 0.97, storage="f32") as b:
         assert b.pop_bytes > 2 ** 32
         start = torch.from_numpy(raw).cuda().view(b.Q, *small[::-1]).repeat(1, *tiles[::-1])
-        b.restore(start.contiguous().view(-1).view(torch.uint8))
+        start = start.contiguous().view(-1).view(torch.uint8)
+        want = want.repeat(1, *tiles[::-1])
+        b.restore(start)
         b.step(2)
         got = b.state_copy().view(torch.float32).view(b.Q, *big[::-1])
-        want = want.repeat(1, *tiles[::-1])
+        assert bool((torch.abs(got - want) <= 4e-6 * torch.abs(want)).all())
+    with E.Ensemble(LAT[D], [small, big], [0.97, 0.97], storage="f32") as c:
+        torch.cuda.synchronize()
+        E.elbm_batch_set_populations(c.b, 1, start, E.ELBM_MEM_DEVICE)
+        E.elbm_batch_set_populations(c.b, 0, raw, E.ELBM_MEM_HOST)
+        c.step(2)
+        E.elbm_batch_get_populations(c.b, 1, start, E.ELBM_MEM_DEVICE)
+        c.synchronize()
+        got = start.view(torch.float32).view(3 ** D, *big[::-1])
         assert bool((torch.abs(got - want) <= 4e-6 * torch.abs(want)).all())
 
 
