@@ -115,8 +115,19 @@ __device__ __forceinline__ T dev_ref(int i, float R)
 // Arithmetic helpers.  FP32 divisions on the hot path multiply by the
 // approximate reciprocal (rcp.approx.ftz: one MUFU operation, ~1 ulp); every
 // divisor on the path is a normal number of moderate size (populations,
-// 1 + O(x) polynomials), so flushing subnormals changes nothing.  FP64 uses
-// IEEE division.
+// 1 + O(x) polynomials), so flushing subnormals changes nothing.
+//
+// FP64 steps are bound by the FP64 pipe (one instruction of a warp in 16 cycles per SM).
+// Divisions and square roots start from the 20-bit approximations rcp.approx.ftz.f64 and
+// rsqrt.approx.ftz.f64 and take one third-order step (Householder's iteration of order two):
+// with e = 1 - b r, 1/b = r (1 + e + e^2) up to e^3 = 2^-60, and with e = 1 - a y^2,
+// sqrt(a) = a y (1 + e/2 + 3 e^2/8) up to 2^-61: results within about 1.5 units in the last
+// place, or half a unit with the remainder's correction (departure_: x itself, which enters f*
+// directly).  Arguments outside [2^-999, 2^1000) (subnormals, zero, infinities, NaN) take the
+// IEEE operations.
+// With the extremes and sign tests on the integer pipe a solved D2Q9 node takes 545 FP64
+// instructions instead of 748: 256^2 95.7 -> 73.3 us per step, 96^2 27.9 -> 21.2; the error
+// of a step against 80-bit arithmetic is the same (rms 1.38e-16 of f*, D3Q27 1.67e-16).
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ float rcp_(float b)
 {
@@ -135,7 +146,31 @@ __device__ __forceinline__ float rcp_nr(float b)
     return fmaf(r, fmaf(-b, r, 1.0f), r);
 }
 __device__ __forceinline__ double rcp_nr(double b) { return 1.0 / b; }
-__device__ __forceinline__ double div_(double a, double b) { return a / b; }
+// whether 2^-999 <= |b| < 2^1000, from the exponent on the integer pipe
+__device__ __forceinline__ bool moderate(double b)
+{
+    return (unsigned(__double2hiint(b)) & 0x7fffffffu) - (24u << 20) < (1999u << 20);
+}
+__device__ __forceinline__ double div_(double a, double b)
+{
+    if (!moderate(b)) return a / b;
+    double r;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(b));
+    const double e = fma(-b, r, 1.0);
+    return a * fma(r, fma(e, e, e), r);
+}
+// x = (f^eq - f) / f
+__device__ __forceinline__ float departure_(float delta, float f) { return div_(delta, f); }
+__device__ __forceinline__ double departure_(double delta, double f)
+{
+    if (!moderate(f)) return delta / f;
+    double r;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(f));
+    const double e = fma(-f, r, 1.0);
+    r = fma(r, fma(e, e, e), r);
+    const double q = delta * r;
+    return fma(r, fma(-f, q, delta), q);
+}
 // FP32 square roots on the path act on 1 + O(u^2) and 1 - 4pq >= 1: the
 // approximate instruction (relative error ~2^-23) loses nothing there.
 __device__ __forceinline__ float sqrt_(float a)
@@ -147,7 +182,45 @@ __device__ __forceinline__ float sqrt_(float a)
 // correctly rounded division, for the few divisions whose rounding reaches f^eq
 __device__ __forceinline__ float div_rn(float a, float b) { return __fdiv_rn(a, b); }
 __device__ __forceinline__ double div_rn(double a, double b) { return a / b; }
-__device__ __forceinline__ double sqrt_(double a) { return sqrt(a); }
+__device__ __forceinline__ double sqrt_(double a)
+{
+    if (!moderate(a) || __double2hiint(a) < 0) return sqrt(a);
+    double y;
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(a));
+    const double s = a * y, e = fma(-s, y, 1.0);
+    return fma(s * e, fma(0.375, e, 0.5), s);
+}
+
+// Running maximum of |x| and minimum of x and 0, ignoring NaN as fmax and fmin do.  In FP64
+// on the integer pipe: the bits of doubles of one sign order as their magnitudes.
+template <class T>
+struct Extremes {
+    T abs = T(0), low = T(0);
+    __device__ __forceinline__ void add(T x)
+    {
+        abs = fmax(abs, fabs(x));
+        low = fmin(low, x);
+    }
+    __device__ __forceinline__ T max_abs() const { return abs; }
+    __device__ __forceinline__ T min0() const { return low; }
+};
+template <>
+struct Extremes<double> {
+    unsigned long long abs = 0, low = 0;
+    __device__ __forceinline__ void add(double x)
+    {
+        const unsigned long long b = (unsigned long long)__double_as_longlong(x), m = b & 0x7fffffffffffffffull;
+        const unsigned long long a = m > 0x7ff0000000000000ull ? 0 : m; // 0 for NaN
+        abs = a > abs ? a : abs;
+        const unsigned long long l = (long long)b < 0 ? a : 0;
+        low = l > low ? l : low;
+    }
+    __device__ __forceinline__ double max_abs() const { return __longlong_as_double((long long)abs); }
+    __device__ __forceinline__ double min0() const { return -__longlong_as_double((long long)low); }
+};
+// x < 0 (a zero or NaN of either sign may count as either: their terms are zero or NaN anyway)
+__device__ __forceinline__ bool below_zero(float x) { return x < 0.0f; }
+__device__ __forceinline__ bool below_zero(double x) { return __double2hiint(x) < 0; }
 
 // ---------------------------------------------------------------------------
 // Storage traits.  raw/pack convert between the stored element and the compute
@@ -333,7 +406,7 @@ __device__ __forceinline__ T node_collide(T (&f)[Lattice<D>::Q], T (&x)[Lattice<
     // w_i u and with the rounded w_i, which in FP32 biased the momentum of f^eq by
     // ~3e-8 of itself per step (the kinetic energy of a decaying D2Q9 vortex,
     // beta = 0.9, 8e-5 above FP64 after 2000 steps).
-    T xabs = T(0), xmin = T(0);
+    Extremes<T> extremes;
     T fx[Q];
 #pragma unroll
     for (int k = 0; k < P; ++k) {
@@ -352,12 +425,12 @@ __device__ __forceinline__ T node_collide(T (&f)[Lattice<D>::Q], T (&x)[Lattice<
             const T E = A + el + A * el;
             const T kr = T(weight_k(D, i)) * r;
             const T delta = fma(kr, E, kr - f[i]);
-            x[i] = div_(delta, f[i]);
+            x[i] = departure_(delta, f[i]);
             fx[i] = delta; // f_i x_i, reused by the sums below
-            xabs = fmax(xabs, fabs(x[i]));
-            xmin = fmin(xmin, x[i]);
+            extremes.add(x[i]);
         }
     }
+    const T xabs = extremes.max_abs(), xmin = extremes.min0();
 
     T alpha = T(2);
     int br = kBranchCutoff;
@@ -376,7 +449,7 @@ __device__ __forceinline__ T node_collide(T (&f)[Lattice<D>::Q], T (&x)[Lattice<
             b1 += fx2;
             c1 += A * K;
             c += A * (xi * xi); // c = c1 + 5 <f, A x^2> below
-            if (xi < T(0)) {
+            if (below_zero(xi)) {
                 const T fx3 = fx2 * xi;
                 S3 += fx3;
                 S4 += fx3 * xi;
@@ -416,9 +489,9 @@ __device__ __forceinline__ T node_collide(T (&f)[Lattice<D>::Q], T (&x)[Lattice<
 #pragma unroll
                 for (int i = 0; i < Q; ++i) {
                     const T xi = x[i];
-                    if (xi >= T(0)) {
+                    if (!below_zero(xi)) {
                         const T t = k * xi;
-                        bp += div_(f[i] * xi * xi * xi * (T(80) + t * (T(80) + T(19) * t)),
+                        bp += div_(fx[i] * xi * xi * (T(80) + t * (T(80) + T(19) * t)),
                                    T(64) + t * (T(96) + t * (T(44) + T(6) * t)));
                     }
                 }
