@@ -68,15 +68,16 @@ __device__ __forceinline__ void node_coords(int64_t n, const Geometry &g, int &x
 // nodes per thread (D2Q9): blocks along x-rows, y = blockIdx.y; byte offsets there are 55.8
 // against 59.0 us per step (2048^2 FP32, developed flow) and 24.6 against 26.5 (1501 x 997,
 // FP32 and FP16 deviations), and leave the DRAM-bound shear layers as they were.
-// Minimum resident blocks per SM requested from the register allocator for the
-// direct step kernel.  D3Q27 with FP32 storage: 7 blocks of 128 (72 registers).
-// Near equilibrium the step is bound by load latency, and the extra resident warps
-// outweigh the spills, which fall in the per-population form of the coefficients
-// (large |x| only): 0.640 -> 0.627 ms per 256^3 step on GB300.  The 16-bit storages
-// lose with that cap (their loads and stores need more live values): 5 blocks, the
-// allocation they had unbounded.  FP32 deviations (d_i kept, f_i formed again at each
-// use): 6 blocks of 128 (80 registers; 0.6375 against 0.6574 ms early at 7).  FP64 (the
-// parity path): no bound.
+// Minimum resident blocks per SM requested from the register allocator for the direct step
+// kernel.  D3Q27 with FP32 storage: 7 blocks of 128 (72 registers).  A step from DRAM is bound
+// by the bytes in flight, and the extra resident warps outweigh the spills (256^3, Taylor-Green
+// start: 0.544 ms with 7 blocks, 0.551 with 6, 0.579 with 5, 0.566 with 8).  FP32 deviations: 6
+// (80 registers).  A step whose two buffers stay in the L2 is bound by instructions and latency
+// instead: 5 blocks there (kL2Blocks, up to 102 registers, no spills; us per step, 7 or 6 blocks
+// and 5, near-equilibrium and developed flow: FP32 32^3 3.20, 3.04 and 3.33, 3.07; 64^3 10.96,
+// 10.45 and 14.69, 14.01; 80^3 20.7, 20.5 and 27.5, 26.4; 96^3, beyond the L2, 34.1, 35.3 and
+// 44.8, 43.5; FP32 deviations 32^3 3.54, 3.24, 72^3 16.2, 15.2 and 21.6, 20.8).  The 16-bit
+// storages take 5 everywhere, the allocation they had unbounded.  FP64: no bound.
 // ELBM_STEP_MIN_BLOCKS overrides.
 #ifndef ELBM_STEP_MIN_BLOCKS
 #define ELBM_STEP_MIN_BLOCKS 0
@@ -113,7 +114,9 @@ constexpr int step_threads()
 {
     return kStepBlock / nodes_per_thread<D, ST>();
 }
-#define ELBM_STEP_BOUNDS __launch_bounds__(step_threads<ST>(), step_min_blocks<ST>())
+constexpr int kL2Blocks = 5;
+// Bytes of the two population buffers up to which a step is taken to run from the L2 (129 MB).
+constexpr uint64_t kL2Bytes = 112ull << 20;
 
 enum { kAddrBytes = 0, kAddrElems = 1, kAddrWide = 2 };
 
@@ -224,8 +227,8 @@ __device__ __forceinline__ void step1_node(const typename ST::S *in, typename ST
     for (int i = 0; i < Q; ++i) __stcs(at<kAddr>(out, uint32_t(i) * N * B + n), ST::pack(f[i]));
 }
 
-template <class ST, int kAddr, bool kForce = false>
-__global__ void ELBM_STEP_BOUNDS k_step(const typename ST::S *__restrict__ fin,
+template <class ST, int kAddr, bool kForce = false, int kBlocks = step_min_blocks<ST>()>
+__global__ void __launch_bounds__(step_threads<ST>(), kBlocks) k_step(const typename ST::S *__restrict__ fin,
                                                     typename ST::S *__restrict__ fout, Geometry g,
                                                     CollideParams p, RowDiv rd)
 {
@@ -1676,6 +1679,16 @@ cudaError_t ELBM_CAT(launch_step, ELBM_SUFFIX)(int storage, const void *fin, voi
             while (threads > 32 && int64_t(blocks_for(plane, threads)) * g.nz < 2 * int64_t(num_sms)) threads /= 2;
         const dim3 grid = pair ? dim3(blocks_for(g.nx, kStepBlock), unsigned(g.ny))
                                : dim3(blocks_for(plane, threads), unsigned(g.nz));
+        if constexpr (D == 3) { // the tighter register bounds are for DRAM
+            if (!forced && 2 * elems * storage_bytes(storage) <= kL2Bytes) {
+#define ELBM_L2_STEP(STT)                                                                              \
+    return launch(k_step<STT, kAddrBytes, false, kL2Blocks>, grid, threads, s,                         \
+                  static_cast<const float *>(fin), static_cast<float *>(fout), g, p, rd)
+                if (storage == ELBM_STORE_F32) ELBM_L2_STEP(StoreF32);
+                if (storage == ELBM_STORE_F32DEV) ELBM_L2_STEP(StoreF32Dev);
+#undef ELBM_L2_STEP
+            }
+        }
         if (elems * storage_bytes(storage) <= 0xffffffffull) {
             ELBM_DIRECT_STEP(kAddrBytes, grid)
         } else {
