@@ -179,9 +179,6 @@ __device__ __forceinline__ float sqrt_(float a)
     asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(a));
     return r;
 }
-// correctly rounded division, for the few divisions whose rounding reaches f^eq
-__device__ __forceinline__ float div_rn(float a, float b) { return __fdiv_rn(a, b); }
-__device__ __forceinline__ double div_rn(double a, double b) { return a / b; }
 __device__ __forceinline__ double sqrt_(double a)
 {
     if (!moderate(a) || __double2hiint(a) < 0) return sqrt(a);
@@ -225,8 +222,8 @@ __device__ __forceinline__ bool below_zero(double x) { return __double2hiint(x) 
 // ---------------------------------------------------------------------------
 // Storage traits.  raw/pack convert between the stored element and the compute
 // type as they are (populations, or deviations d_i = f_i - c_i where kDev);
-// load/store (and load64/store64 for FP64 companions) take the reference c_i of
-// population i and convert to and from populations f_i.  The step kernels load
+// load (and load64/store64 in FP64) takes the reference c_i of population i and converts to
+// (and from) populations f_i.  The step kernels load
 // with raw, hand the stored values to collide_stored and store with pack: the
 // collision works on the deviations themselves where kDevCollide (FP32 deviations,
 // so that no rounding happens at the scale of w_i), and on populations formed from
@@ -241,7 +238,6 @@ struct StoreF64 {
     __device__ static __forceinline__ T raw(S s) { return s; }
     __device__ static __forceinline__ S pack(T v) { return v; }
     __device__ static __forceinline__ T load(S s, T) { return s; }
-    __device__ static __forceinline__ S store(T f, T) { return f; }
     __device__ static __forceinline__ double load64(S s, double) { return s; }
     __device__ static __forceinline__ S store64(double f, double) { return f; }
 };
@@ -253,7 +249,6 @@ struct StoreF32 {
     __device__ static __forceinline__ T raw(S s) { return s; }
     __device__ static __forceinline__ S pack(T v) { return v; }
     __device__ static __forceinline__ T load(S s, T) { return s; }
-    __device__ static __forceinline__ S store(T f, T) { return f; }
     __device__ static __forceinline__ double load64(S s, double) { return double(s); }
     __device__ static __forceinline__ S store64(double f, double) { return float(f); }
 };
@@ -265,7 +260,6 @@ struct StoreF32Dev {
     __device__ static __forceinline__ T raw(S s) { return s; }
     __device__ static __forceinline__ S pack(T v) { return v; }
     __device__ static __forceinline__ T load(S s, T c) { return c + s; }
-    __device__ static __forceinline__ S store(T f, T c) { return f - c; }
     __device__ static __forceinline__ double load64(S s, double c) { return c + double(s); }
     __device__ static __forceinline__ S store64(double f, double c) { return float(f - c); }
 };
@@ -277,7 +271,6 @@ struct StoreF16Dev {
     __device__ static __forceinline__ T raw(S s) { return __half2float(s); }
     __device__ static __forceinline__ S pack(T v) { return __float2half_rn(v); }
     __device__ static __forceinline__ T load(S s, T c) { return c + raw(s); }
-    __device__ static __forceinline__ S store(T f, T c) { return pack(f - c); }
     __device__ static __forceinline__ double load64(S s, double c) { return c + double(__half2float(s)); }
     __device__ static __forceinline__ S store64(double f, double c) { return __double2half(f - c); }
 };
@@ -289,7 +282,6 @@ struct StoreBF16Dev {
     __device__ static __forceinline__ T raw(S s) { return __bfloat162float(s); }
     __device__ static __forceinline__ S pack(T v) { return __float2bfloat16_rn(v); }
     __device__ static __forceinline__ T load(S s, T c) { return c + raw(s); }
-    __device__ static __forceinline__ S store(T f, T c) { return pack(f - c); }
     __device__ static __forceinline__ double load64(S s, double c) { return c + double(__bfloat162float(s)); }
     __device__ static __forceinline__ S store64(double f, double c) { return __double2bfloat16(f - c); }
 };

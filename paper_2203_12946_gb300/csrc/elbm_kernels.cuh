@@ -1001,6 +1001,7 @@ __global__ void __launch_bounds__(kStepBlock, step_diag_min_blocks<ST>()) k_step
 }
 
 // --------------------------------------------------------------------------
+#if ELBM_DIM == 2
 // --------------------------------------------------------------------------
 // Several steps of a small D2Q9 domain in one launch.  A step of a small domain costs its
 // latency, not its work: the launch, one pull from L2, one pass through the collision's chain
@@ -1078,6 +1079,7 @@ __global__ void __launch_bounds__(kTileThreads, 1) k_step_tile(const typename ST
         if (step < k) __syncthreads();
     }
 }
+#endif
 
 // --------------------------------------------------------------------------
 // Batched ensemble: one launch advances up to kBatchTableDomains domains.  Block
@@ -1498,11 +1500,11 @@ __global__ void __launch_bounds__(kAuxBlock) k_equilibrium_vjp(const double *__r
 // --------------------------------------------------------------------------
 #define ELBM_STORAGE_SWITCH(storage, CALL)                                                     \
     switch (storage) {                                                                         \
-    case ELBM_STORE_F64: { using ST = StoreF64; CALL; break; }                                 \
-    case ELBM_STORE_F32: { using ST = StoreF32; CALL; break; }                                 \
-    case ELBM_STORE_F32DEV: { using ST = StoreF32Dev; CALL; break; }                           \
-    case ELBM_STORE_F16DEV: { using ST = StoreF16Dev; CALL; break; }                           \
-    case ELBM_STORE_BF16DEV: { using ST = StoreBF16Dev; CALL; break; }                         \
+    case ELBM_STORE_F64: { using ST = StoreF64; CALL; }                                        \
+    case ELBM_STORE_F32: { using ST = StoreF32; CALL; }                                        \
+    case ELBM_STORE_F32DEV: { using ST = StoreF32Dev; CALL; }                                  \
+    case ELBM_STORE_F16DEV: { using ST = StoreF16Dev; CALL; }                                  \
+    case ELBM_STORE_BF16DEV: { using ST = StoreBF16Dev; CALL; }                                \
     default: return cudaErrorInvalidValue;                                                     \
     }
 
@@ -1517,7 +1519,7 @@ static inline unsigned blocks_for(int64_t N, int block) { return unsigned((N + b
 #define ELBM_CAT2(a, b) a##_##b
 #define ELBM_CAT(a, b) ELBM_CAT2(a, b)
 
-// A lattice may be compiled in three units: ELBM_PART 1 holds the step launcher (and the
+// Each lattice is compiled in three units: ELBM_PART 1 holds the step launcher (and the
 // row pipeline), ELBM_PART 3 the launchers of the batched ensemble, ELBM_PART 2 every other
 // launcher; without ELBM_PART one unit holds all.
 #if !defined(ELBM_PART) || ELBM_PART == 1
@@ -1630,11 +1632,11 @@ cudaError_t ELBM_CAT(launch_step, ELBM_SUFFIX)(int storage, const void *fin, voi
     if (kernel == ELBM_KERNEL_ROWS) return cudaErrorNotSupported;
     if (steps > 1) {
         if (steps > ELBM_CAT(steps_per_launch, ELBM_SUFFIX)(storage, g, kernel, num_sms)) return cudaErrorInvalidValue;
-        if constexpr (D == 2) {
-            const unsigned R = unsigned(kTileRows + 2 * (steps - 1)), nx = unsigned(g.nx);
-            const unsigned threads = R * ((nx + kPairSpan - 1) / kPairSpan) * 32u; // at most kTileThreads
-            const size_t shared = size_t(Q) * (R + R - 2) * nx * storage_bytes(storage);
-            const unsigned grid = unsigned((g.ny + kTileRows - 1) / kTileRows);
+#if ELBM_DIM == 2
+        const unsigned R = unsigned(kTileRows + 2 * (steps - 1)), nx = unsigned(g.nx);
+        const unsigned threads = R * ((nx + kPairSpan - 1) / kPairSpan) * 32u; // at most kTileThreads
+        const size_t shared = size_t(Q) * (R + R - 2) * nx * storage_bytes(storage);
+        const unsigned grid = unsigned((g.ny + kTileRows - 1) / kTileRows);
 #define ELBM_TILE(FORCE)                                                                                    \
     switch (storage) {                                                                                      \
     case ELBM_STORE_F32: { using ST = StoreF32; ELBM_TILE_ONE(FORCE); }                                     \
@@ -1646,11 +1648,11 @@ cudaError_t ELBM_CAT(launch_step, ELBM_SUFFIX)(int storage, const void *fin, voi
     return launch_shared(k_step_tile<ST, FORCE>, grid, threads, shared, s,                                  \
                          static_cast<const typename ST::S *>(fin), static_cast<typename ST::S *>(fout), g,  \
                          p, steps, kTileRows)
-            if (forced) ELBM_TILE(true)
-            ELBM_TILE(false)
+        if (forced) ELBM_TILE(true)
+        ELBM_TILE(false)
 #undef ELBM_TILE
 #undef ELBM_TILE_ONE
-        }
+#endif
     }
     const uint64_t elems = uint64_t(Q) * uint64_t(g.N);
     const RowDiv rd = row_div(uint32_t(g.nx));
@@ -1679,16 +1681,16 @@ cudaError_t ELBM_CAT(launch_step, ELBM_SUFFIX)(int storage, const void *fin, voi
             while (threads > 32 && int64_t(blocks_for(plane, threads)) * g.nz < 2 * int64_t(num_sms)) threads /= 2;
         const dim3 grid = pair ? dim3(blocks_for(g.nx, kStepBlock), unsigned(g.ny))
                                : dim3(blocks_for(plane, threads), unsigned(g.nz));
-        if constexpr (D == 3) { // the tighter register bounds are for DRAM
-            if (!forced && 2 * elems * storage_bytes(storage) <= kL2Bytes) {
+#if ELBM_DIM == 3 // the tighter register bounds are for DRAM
+        if (!forced && 2 * elems * storage_bytes(storage) <= kL2Bytes) {
 #define ELBM_L2_STEP(STT)                                                                              \
     return launch(k_step<STT, kAddrBytes, false, kL2Blocks>, grid, threads, s,                         \
-                  static_cast<const float *>(fin), static_cast<float *>(fout), g, p, rd)
-                if (storage == ELBM_STORE_F32) ELBM_L2_STEP(StoreF32);
-                if (storage == ELBM_STORE_F32DEV) ELBM_L2_STEP(StoreF32Dev);
+              static_cast<const float *>(fin), static_cast<float *>(fout), g, p, rd)
+            if (storage == ELBM_STORE_F32) ELBM_L2_STEP(StoreF32);
+            if (storage == ELBM_STORE_F32DEV) ELBM_L2_STEP(StoreF32Dev);
 #undef ELBM_L2_STEP
-            }
         }
+#endif
         if (elems * storage_bytes(storage) <= 0xffffffffull) {
             ELBM_DIRECT_STEP(kAddrBytes, grid)
         } else {
@@ -1696,7 +1698,6 @@ cudaError_t ELBM_CAT(launch_step, ELBM_SUFFIX)(int storage, const void *fin, voi
         }
     }
 #undef ELBM_DIRECT_STEP
-    return cudaGetLastError();
 }
 
 #endif
@@ -1716,7 +1717,6 @@ cudaError_t ELBM_CAT(launch_step_diag, ELBM_SUFFIX)(int storage, const void *fin
     ELBM_STORAGE_SWITCH(storage, return launch(k_step_diag<ST>, grid, kStepBlock, s,
                                                static_cast<const typename ST::S *>(fin),
                                                static_cast<typename ST::S *>(fout), g, p, acc))
-    return cudaGetLastError();
 }
 
 #endif
@@ -1858,7 +1858,6 @@ cudaError_t ELBM_CAT(launch_kinetic_energy, ELBM_SUFFIX)(int storage, const void
     ELBM_STORAGE_SWITCH(storage, return launch(k_kinetic_energy<ST>, blocks, kAuxBlock, s,
                                                static_cast<const typename ST::S *>(f), g, Rf, Rsum, acc,
                                                static_cast<typename ST::T *>(grad)))
-    return cudaGetLastError();
 }
 
 cudaError_t ELBM_CAT(launch_equilibrium_vjp, ELBM_SUFFIX)(int storage, const double *rho, const double *u,
@@ -1883,7 +1882,6 @@ cudaError_t ELBM_CAT(launch_init, ELBM_SUFFIX)(int storage, const double *rho, c
     ELBM_STORAGE_SWITCH(storage, return launch(k_init<ST>, blocks_for(count, kAuxBlock), kAuxBlock, s, rho,
                                                u, static_cast<typename ST::S *>(f), g, rho_uniform, rho0, n0,
                                                count))
-    return cudaGetLastError();
 }
 
 cudaError_t ELBM_CAT(launch_moments, ELBM_SUFFIX)(int storage, const void *f, const Geometry &g,
@@ -1897,7 +1895,6 @@ cudaError_t ELBM_CAT(launch_moments, ELBM_SUFFIX)(int storage, const void *f, co
     ELBM_STORAGE_SWITCH(storage, return launch(k_moments<ST>, blocks_for(count, kAuxBlock), kAuxBlock, s,
                                                static_cast<const typename ST::S *>(f), g, Rf, Rsum, rho_out,
                                                u_out, n0, count))
-    return cudaGetLastError();
 }
 
 cudaError_t ELBM_CAT(launch_alpha, ELBM_SUFFIX)(int storage, const void *f, const Geometry &g,
@@ -1909,7 +1906,6 @@ cudaError_t ELBM_CAT(launch_alpha, ELBM_SUFFIX)(int storage, const void *f, cons
     ELBM_STORAGE_SWITCH(storage, return launch(k_alpha<ST>, blocks_for(g.N, kStepBlock), kStepBlock, s,
                                                static_cast<const typename ST::S *>(f), g, p, alpha_out,
                                                flags, nut_out))
-    return cudaGetLastError();
 }
 
 cudaError_t ELBM_CAT(launch_diag, ELBM_SUFFIX)(int storage, const void *f, const Geometry &g,
@@ -1923,7 +1919,6 @@ cudaError_t ELBM_CAT(launch_diag, ELBM_SUFFIX)(int storage, const void *f, const
     if (blocks > cap) blocks = cap;
     ELBM_STORAGE_SWITCH(storage, return launch(k_diag<ST>, blocks, kAuxBlock, s,
                                                static_cast<const typename ST::S *>(f), g, p, acc))
-    return cudaGetLastError();
 }
 
 #endif
