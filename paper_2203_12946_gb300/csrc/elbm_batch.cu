@@ -47,7 +47,7 @@ struct elbm_batch {
     size_t total_elems = 0;   // elements per buffer
     void *pop[2] = {nullptr, nullptr};
     int cur = 0;
-    int bx = 128;                          // work-item width (autotuned)
+    int bx = 0;                            // work-item width (autotuned; at first default_width)
     std::map<int, std::vector<eelbm::BatchTable>> tables; // per width: the launches of one batched step
     double *stage = nullptr;
     size_t stage_bytes = 0;
@@ -150,6 +150,13 @@ int check_domain(elbm_batch_t *b, int d, const char *what)
         return bfail(b, ELBM_ERR_ARG, "%s: domain %d out of range [0, %d)", what, d, int(b->doms.size()));
     return ELBM_OK;
 }
+
+// Work-item width before elbm_batch_tune.  D2Q9: 64, the 64 nodes of one warp (us per step with
+// 64, 128, 256 nodes, FP32: 64 domains of sides 64 to 512 73.9, 76.5, 78.8; 64 of 64^2 6.6, 9.5,
+// 8.7; 64 of 192^2 34.1, 44.0, 35.3; 16 of 300 x 200 19.0, 22.3, 20.9; 32 of 512^2 132, 133, 133):
+// wider blocks hold idle warps wherever the width does not divide a row.  D3Q27: 128 (one node
+// per thread; 16 of 32^3 54.1, 39.9, 136; 6 of 100 x 60 x 50 116, 115, 176).
+int default_width(int D) { return D == 2 ? 64 : 128; }
 
 // Parameter tables of the batched launches of width bx: consecutive runs of up to
 // kBatchTableDomains domains, one launch each.
@@ -397,6 +404,7 @@ int elbm_batch_create(elbm_batch_t **out, int lattice, int ndomains, const int64
     if (!b) return bfail(nullptr, ELBM_ERR_ARG, "elbm_batch_create: out of host memory");
     b->lattice = lattice;
     b->D = lattice == ELBM_D2Q9 ? 2 : 3;
+    b->bx = default_width(b->D);
     b->Q = Q;
     b->opts = o;
     b->doms = doms;
