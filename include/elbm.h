@@ -200,8 +200,8 @@ int elbm_set_stream(elbm_t *h, void *stream);
 
 /* Initial state f = f^eq(rho, u) at every node (Sec. I equilibrium), computed
  * in FP64 (for the FP32 and 16-bit storages in double-length FP32 arithmetic of
- * ~44 bits, and for FP32 deviations in FP64 where that could change the last bit)
- * and rounded to the storage type.  rho: N doubles (NULL = uniform rho0); u:
+ * ~44 bits, and for deviations in FP64 where that could change the last bit)
+ * and rounded once to the storage type.  rho: N doubles (NULL = uniform rho0); u:
  * D*N doubles, u[a*N + n].  where = ELBM_MEM_DEVICE or ELBM_MEM_HOST (host
  * arrays are copied through a library-owned staging buffer, in node ranges
  * that overlap the copies with the computation; the first host call creates

@@ -266,6 +266,7 @@ struct StoreF32Dev {
 struct StoreF16Dev {
     using S = __half;
     using T = float;
+    static constexpr int kBits = 11, kMinExponent = 113; // significant bits; 2^-14 in FP32's bias
     static constexpr bool kDev = true, kDevCollide = false;
     static constexpr int kRows = 1;
     __device__ static __forceinline__ T raw(S s) { return __half2float(s); }
@@ -277,6 +278,7 @@ struct StoreF16Dev {
 struct StoreBF16Dev {
     using S = __nv_bfloat16;
     using T = float;
+    static constexpr int kBits = 8, kMinExponent = 1;
     static constexpr bool kDev = true, kDevCollide = false;
     static constexpr int kRows = 1;
     __device__ static __forceinline__ T raw(S s) { return __bfloat162float(s); }

@@ -393,14 +393,26 @@ __device__ __forceinline__ DF df_sqrt(DF a)
     return df_fast_two_sum(r, e / (2.0f * r));
 }
 
-// The equilibrium in double-float, less k_i R (R = 0: populations), rounded once to FP32:
-// |error| <= half an FP32 ulp + about 2^-44 f^eq.  Per axis phi(-1) = Y den / (6 num) and
-// phi(+1) = Y num / (6 den) share one division, r = Y / (6 num den), phi(-1) = r den^2,
-// phi(+1) = r num^2.  Returns whether every value is known to be the correctly rounded one
-// (only with kSure: f^eq - k_i R is small, so 2^-44 f^eq can reach its last bit): the error
-// term of the sum is further than 2^-44 f^eq from half an ulp of the result.
-template <bool kSure>
-__device__ __forceinline__ bool equilibrium_df(DF rho, const DF (&u)[3], float R, float (&feq)[Q])
+// v + err, where |err| is at most half a unit in the last place of v, rounded to odd: v if the
+// sum is exact or v is odd, else v's odd neighbour on the side of err.  The 13 or more bits that
+// a conversion to 16 bits then drops still tell on which side of a midpoint the sum lies, so
+// that the conversion rounds the sum itself (Boldo and Melquiond, Emulation of FMA and correctly
+// rounded sums, 2008).
+__device__ __forceinline__ float to_odd(float v, float err)
+{
+    const uint32_t b = __float_as_uint(v);
+    if (err == 0.0f || (b & 1u)) return v;
+    return __uint_as_float((err < 0.0f) == (v < 0.0f) ? b + 1u : b - 1u);
+}
+
+// The equilibrium in double-float, less k_i R (R = 0: populations), rounded once to the storage:
+// |error| <= half a unit in the last place + about 2^-44 f^eq.  Per axis phi(-1) = Y den / (6 num)
+// and phi(+1) = Y num / (6 den) share one division, r = Y / (6 num den), phi(-1) = r den^2,
+// phi(+1) = r num^2.  Returns whether every value is known to be the correctly rounded one (asked
+// of the deviations only: f^eq - k_i R is small, so 2^-44 f^eq can reach its last bit): what the
+// stored value leaves of the sum is further than 2^-44 f^eq from half a unit in its last place.
+template <class ST>
+__device__ __forceinline__ bool equilibrium_df(DF rho, const DF (&u)[3], float R, typename ST::S (&feq)[Q])
 {
     constexpr double kTwoThirds = 2.0 / 3.0;
     const DF two3 = {float(kTwoThirds), float(kTwoThirds - double(float(kTwoThirds)))};
@@ -432,16 +444,24 @@ __device__ __forceinline__ bool equilibrium_df(DF rho, const DF (&u)[3], float R
     const DF b0 = phi[D - 1][0], b1 = phi[D - 1][1], b2 = phi[D - 1][2];
     const float2 bh = f2(b0.hi, b2.hi), bl = f2(b0.lo, b2.lo);
     auto put = [&](int i, float p, float en) {
-        const float c = -float(weight_k(D, i)) * R, d = p + c;
-        if constexpr (kSure) {
-            const float dd = d - p;
+        if constexpr (!ST::kDev) {
+            feq[i] = ST::pack(p - en);
+        } else {
+            const float c = -float(weight_k(D, i)) * R, d = p + c, dd = d - p;
             const float w = ((p - (d - dd)) + (c - dd)) - en; // what p + c - d lost, and p's error
             const float r1 = d + w, err = w - (r1 - d);
-            const float half_ulp = __uint_as_float(max(__float_as_uint(r1) & 0x7f800000u, 24u << 23) - (24u << 23));
-            sure = sure && fabsf(fabsf(err) - half_ulp) > 0x1p-44f * p;
-            feq[i] = r1;
-        } else {
-            feq[i] = d - en;
+            const uint32_t expo = __float_as_uint(r1) & 0x7f800000u;
+            float gap; // what the stored value leaves of the sum, less half a unit in its last place
+            if constexpr (sizeof(typename ST::S) == 4) {
+                feq[i] = ST::pack(r1);
+                gap = fabsf(err) - __uint_as_float(max(expo, 24u << 23) - (24u << 23));
+            } else {
+                constexpr uint32_t bits = ST::kBits, low = ST::kMinExponent;
+                feq[i] = ST::pack(to_odd(r1, err));
+                const float t = r1 - ST::raw(feq[i]);
+                gap = (fabsf(t) - __uint_as_float(max(expo, max(low, bits + 1u) << 23) - (bits << 23))) + (t < 0.0f ? -err : err);
+            }
+            sure = sure && fabsf(gap) > 0x1p-44f * p;
         }
     };
 #pragma unroll
@@ -458,12 +478,13 @@ __device__ __forceinline__ bool equilibrium_df(DF rho, const DF (&u)[3], float R
 }
 
 // f = f^eq(rho, u) for the nodes n0 .. n0 + count - 1 (SoA with stride g.N).  FP64 storage
-// in FP64; the FP32-arithmetic storages in double-float (equilibrium_df), rounded once to
-// FP32 (then to 16 bits), but for a node whose FP32 deviations are not sure to be rounded as
-// FP64 would (a few nodes in a hundred): FP64 again.  4.8 M D3Q27 nodes: 145 us for FP32
-// populations (158 with FP64 conversions), 228 for FP32 deviations and 151 for FP16 (1 433 in
-// FP64); 8 M D2Q9 nodes: 133, 171 and 138 (184, 1 249, 1 250).  Bound by the FP32 arithmetic and
-// its issue slots.  The factors without divisions (1 + 2t -+ 3u) take 122 and 108 us, but round
+// in FP64; the FP32-arithmetic storages in double-float (equilibrium_df), rounded once, but for
+// a node whose deviations are not sure to be rounded as FP64 would (FP32: a few nodes in a
+// hundred, 16 bits: one in millions): FP64 again.  4.8 M D3Q27 nodes: 145 us for FP32
+// populations (158 with FP64 conversions), 228 for FP32 deviations and 254 for FP16 (1 433 in
+// FP64; 151 when FP16 is rounded twice, first to FP32, which gives another value at 6 in 10^5);
+// 8 M D2Q9 nodes: 133, 171 and 188 (184, 1 249, 1 250).  Bound by the FP32 arithmetic and its
+// issue slots.  The factors without divisions (1 + 2t -+ 3u) take 122 and 108 us, but round
 // a few values in 10^8 the other way than this form, which would show in FP64 moments.
 template <class ST>
 __global__ void __launch_bounds__(kAuxBlock) k_init(const double *__restrict__ rho,
@@ -481,12 +502,10 @@ __global__ void __launch_bounds__(kAuxBlock) k_init(const double *__restrict__ r
     for (int a = 0; a < D; ++a) un[a] = __ldcs(u + (int64_t)a * g.N + n);
     if constexpr (sizeof(typename ST::T) == 4) {
         const DF ud[3] = {df_from_double(un[0]), df_from_double(un[1]), df_from_double(un[2])};
-        float fe[Q];
-        const float R = ST::kDev ? dev_unit<D>(rho0) : 0.0f;
-        const bool sure = equilibrium_df<ST::kDevCollide>(df_from_double(r), ud, R, fe);
-        if (!ST::kDevCollide || sure) {
+        typename ST::S fe[Q];
+        if (equilibrium_df<ST>(df_from_double(r), ud, ST::kDev ? dev_unit<D>(rho0) : 0.0f, fe)) {
 #pragma unroll
-            for (int i = 0; i < Q; ++i) f[(int64_t)i * g.N + n] = ST::pack(fe[i]);
+            for (int i = 0; i < Q; ++i) f[(int64_t)i * g.N + n] = fe[i];
             return;
         }
     }
