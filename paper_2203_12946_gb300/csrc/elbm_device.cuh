@@ -121,13 +121,16 @@ __device__ __forceinline__ T dev_ref(int i, float R)
 // Divisions and square roots start from the 20-bit approximations rcp.approx.ftz.f64 and
 // rsqrt.approx.ftz.f64 and take one third-order step (Householder's iteration of order two):
 // with e = 1 - b r, 1/b = r (1 + e + e^2) up to e^3 = 2^-60, and with e = 1 - a y^2,
-// sqrt(a) = a y (1 + e/2 + 3 e^2/8) up to 2^-61: results within about 1.5 units in the last
-// place, or half a unit with the remainder's correction (departure_: x itself, which enters f*
-// directly).  Arguments outside [2^-999, 2^1000) (subnormals, zero, infinities, NaN) take the
-// IEEE operations.
-// With the extremes and sign tests on the integer pipe a solved D2Q9 node takes 545 FP64
-// instructions instead of 748: 256^2 95.7 -> 73.3 us per step, 96^2 27.9 -> 21.2; the error
-// of a step against 80-bit arithmetic is the same (rms 1.38e-16 of f*, D3Q27 1.67e-16).
+// sqrt(a) = a y (1 + e/2 + 3 e^2/8) and 1/sqrt(a) = y (1 + e/2 + 3 e^2/8) up to 2^-61.  Then the
+// remainder a - b q, or a - s^2, of a result within about 2 units in the last place, times 1/b
+// or 1/(2s), is added with one rounding (Markstein, Computation of elementary functions on the
+// IBM RISC System/6000, 1990): the result is the correctly rounded one, unless the exact value
+// lies within 2^-49 of a unit from the middle between two numbers.  Quotients that can (the
+// divisor a unit below a power of two, Markstein's exception) and arguments outside
+// [2^-500, 2^500) (but zero as a numerator) take the IEEE operations.
+// With the extremes and sign tests on the integer pipe, us per step with IEEE operations and
+// comparisons and so: D2Q9 256^2 108.7, 82.4, 96^2 29.3, 24.7, D3Q27 64^3 1012, 797.  Without the
+// remainders (results within 1.5 units): 72.8, 21.1 and 726.
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ float rcp_(float b)
 {
@@ -146,30 +149,22 @@ __device__ __forceinline__ float rcp_nr(float b)
     return fmaf(r, fmaf(-b, r, 1.0f), r);
 }
 __device__ __forceinline__ double rcp_nr(double b) { return 1.0 / b; }
-// whether 2^-999 <= |b| < 2^1000, from the exponent on the integer pipe
+// whether 2^-500 <= |b| < 2^500, from the exponent on the integer pipe; with kZero also for zero
+template <bool kZero = false>
 __device__ __forceinline__ bool moderate(double b)
 {
-    return (unsigned(__double2hiint(b)) & 0x7fffffffu) - (24u << 20) < (1999u << 20);
+    const unsigned m = unsigned(__double2hiint(b)) & 0x7fffffffu;
+    return m - (523u << 20) < (1000u << 20) || (kZero && (m | unsigned(__double2loint(b))) == 0u);
 }
 __device__ __forceinline__ double div_(double a, double b)
 {
-    if (!moderate(b)) return a / b;
+    if (!(moderate(b) && moderate<true>(a)) || __double2loint(b) == -1) return a / b;
     double r;
     asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(b));
     const double e = fma(-b, r, 1.0);
-    return a * fma(r, fma(e, e, e), r);
-}
-// x = (f^eq - f) / f
-__device__ __forceinline__ float departure_(float delta, float f) { return div_(delta, f); }
-__device__ __forceinline__ double departure_(double delta, double f)
-{
-    if (!moderate(f)) return delta / f;
-    double r;
-    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(f));
-    const double e = fma(-f, r, 1.0);
     r = fma(r, fma(e, e, e), r);
-    const double q = delta * r;
-    return fma(r, fma(-f, q, delta), q);
+    const double q = a * r;
+    return fma(r, fma(-b, q, a), q);
 }
 // FP32 square roots on the path act on 1 + O(u^2) and 1 - 4pq >= 1: the
 // approximate instruction (relative error ~2^-23) loses nothing there.
@@ -184,8 +179,9 @@ __device__ __forceinline__ double sqrt_(double a)
     if (!moderate(a) || __double2hiint(a) < 0) return sqrt(a);
     double y;
     asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(a));
-    const double s = a * y, e = fma(-s, y, 1.0);
-    return fma(s * e, fma(0.375, e, 0.5), s);
+    const double s0 = a * y, h0 = 0.5 * y, r = fma(-s0, h0, 0.5); // r = e/2
+    const double c = fma(1.5 * r, r, r), s = fma(s0, c, s0), h = fma(h0, c, h0);
+    return fma(h, fma(-s, s, a), s);
 }
 
 // Running maximum of |x| and minimum of x and 0, ignoring NaN as fmax and fmin do.  In FP64
@@ -419,7 +415,7 @@ __device__ __forceinline__ T node_collide(T (&f)[Lattice<D>::Q], T (&x)[Lattice<
             const T E = A + el + A * el;
             const T kr = T(weight_k(D, i)) * r;
             const T delta = fma(kr, E, kr - f[i]);
-            x[i] = departure_(delta, f[i]);
+            x[i] = div_(delta, f[i]);
             fx[i] = delta; // f_i x_i, reused by the sums below
             extremes.add(x[i]);
         }

@@ -1,14 +1,84 @@
 """How results are rounded: where a value is formed in more bits than it is stored in, or by a
 division or root of the library's own, it is the correctly rounded one."""
+import ctypes
+import os
+import subprocess
+
 import numpy as np
 import pytest
 
 import oracle as O
+from paper_2203_12946_gb300 import build as B
 from paper_2203_12946_gb300 import elbm as E
 from paper_2203_12946_gb300 import inputs
 from test_gpu_parity import LAT, _cuda, dev_ref  # noqa: F401
 
 pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def probe(tmp_path_factory):
+    """Calls a function of device_probes.cu, built with the library's flags: arrays go in as
+    device copies, the outputs (shape, dtype) come back as arrays."""
+    torch = pytest.importorskip("torch")
+    lib = str(tmp_path_factory.mktemp("probes") / "probes.so")
+    src = os.path.join(os.path.dirname(os.path.abspath(__file__)), "device_probes.cu")
+    subprocess.run([B.nvcc(), *B.ARCH, *B.NVCC_FLAGS, "-shared", "-o", lib, src, "-cudart", "static"], check=True)
+    so = ctypes.CDLL(lib)
+
+    def call(name, ins, outs, *scalars):
+        a = [torch.from_numpy(np.ascontiguousarray(v)).cuda() for v in ins]
+        o = [torch.from_numpy(np.zeros(shape, dtype)).cuda() for shape, dtype in outs]
+        torch.cuda.synchronize()
+        assert getattr(so, name)(*[ctypes.c_void_p(t.data_ptr()) for t in a + o], *scalars) == 0
+        return [t.cpu().numpy() for t in o]
+
+    return call
+
+
+def same(a, b):
+    return np.array_equal(a, b, equal_nan=True)
+
+
+def doubles(rng, n, lo, hi):
+    """Random significands and signs, binary exponents in [lo, hi)."""
+    return np.ldexp(rng.uniform(1.0, 2.0, n), rng.integers(lo, hi, n)) * rng.choice([-1.0, 1.0], n)
+
+
+# around the exponents where the library's forms end, and what they do not take
+EDGES = np.array([0.0, -0.0, 5e-324, 1e-310, 2.0 ** -1022, 2.0 ** -501, 2.0 ** -500, 2.0 ** 500, 2.0 ** 1023,
+                  np.nextafter(2.0 ** -500, 0), np.nextafter(2.0 ** 500, 0), 1.0, np.nextafter(1.0, 0), np.nextafter(2.0, 0),
+                  1.7976931348623157e308, np.inf, np.nan])
+
+
+def test_fp64_division_is_ieee(probe):
+    """The FP64 collision's quotient against the correctly rounded one: the same number wherever
+    the exact quotient is further than 2^-49 of a unit from the middle between two, so at every
+    one of 2^20 random pairs (2^-28 of a chance that one of them is not), and outside the range of
+    the library's form, which leaves those to the IEEE operation."""
+    rng = np.random.default_rng(1)
+    n = 1 << 18
+    e = np.concatenate([EDGES, -EDGES, doubles(rng, 40, -520, -480), doubles(rng, 40, 480, 520)])
+    a = np.concatenate([doubles(rng, n, -3, 3), doubles(rng, n, -60, 4), doubles(rng, n, -520, 520), doubles(rng, n, -1074, 1024),
+                        np.repeat(e, e.size)])
+    b = np.concatenate([doubles(rng, n, -3, 3), doubles(rng, n, -12, 8), doubles(rng, n, -520, 520), doubles(rng, n, -1074, 1024),
+                        np.tile(e, e.size)])
+    out, ieee = probe("probe_div", [a, b], [(a.shape, np.float64)] * 2, a.size)
+    with np.errstate(all="ignore"):
+        assert same(ieee, a / b)
+    assert same(out, ieee)
+
+
+def test_fp64_square_root_is_ieee(probe):
+    """As test_fp64_division_is_ieee: 1/(2s) here is good to 2^-50."""
+    rng = np.random.default_rng(2)
+    n = 1 << 19
+    e = np.concatenate([EDGES, -EDGES])
+    a = np.concatenate([rng.uniform(1.0, 1.2, n), np.abs(doubles(rng, n, -520, 520)), np.abs(doubles(rng, n, -1074, 1024)), e])
+    out, ieee = probe("probe_sqrt", [a], [(a.shape, np.float64)] * 2, a.size)
+    with np.errstate(all="ignore"):
+        assert same(ieee, np.sqrt(a))
+    assert same(out, ieee)
 
 
 @pytest.mark.parametrize("storage", ["f16dev", "bf16dev"])
