@@ -514,18 +514,13 @@ __device__ __forceinline__ bool node_vjp_series(const float (&F)[Lattice<D>::Q],
     // alpha and the adjoints m_k, s_k of the power sums
     float alpha = 2.0f, m2 = 0.0f, m3 = 0.0f, m4 = 0.0f, m5 = 0.0f, m6 = 0.0f, s3 = 0.0f, s4 = 0.0f, s5 = 0.0f, s6 = 0.0f;
     if (!lbgk && !(p.cutoff && xabs < float(kCutoff))) {
-        float2 M2 = f2(0.0f), M3 = f2(0.0f), M4 = f2(0.0f), M5 = f2(0.0f), M6 = f2(0.0f);
-        float2 A3 = f2(0.0f), A4 = f2(0.0f), A5 = f2(0.0f), A6 = f2(0.0f);
+        PowerSums sums;
 #pragma unroll
-        for (int k = 0; k < NP; ++k) {
-            const float2 x2 = pmul(x[k], x[k]), g2 = pmul(f[k], x2), g4 = pmul(g2, x2);
-            const float2 axk = f2(fabsf(x[k].x), fabsf(x[k].y)), xax = pmul(x[k], axk);
-            M2 = padd(M2, g2), M3 = pfma(g2, x[k], M3), M4 = padd(M4, g4), M5 = pfma(g4, x[k], M5), M6 = pfma(g4, x2, M6);
-            A3 = pfma(g2, axk, A3), A4 = pfma(g2, xax, A4), A5 = pfma(g4, axk, A5), A6 = pfma(g4, xax, A6);
-        }
-        const float S2 = M2.x + M2.y, T3 = M3.x + M3.y, T4 = M4.x + M4.y, T5 = M5.x + M5.y, T6 = M6.x + M6.y;
-        const float S3 = 0.5f * (T3 - (A3.x + A3.y)), S4 = 0.5f * (T4 - (A4.x + A4.y));
-        const float S5 = 0.5f * (T5 - (A5.x + A5.y)), S6 = 0.5f * (T6 - (A6.x + A6.y));
+        for (int k = 0; k < NP; ++k) sums.add(f[k], x[k]);
+        const float S2 = sums.M2.x + sums.M2.y, T3 = sums.M3.x + sums.M3.y, T4 = sums.M4.x + sums.M4.y;
+        const float T5 = sums.M5.x + sums.M5.y, T6 = sums.M6.x + sums.M6.y;
+        const float S3 = sums.S3.x + sums.S3.y, S4 = sums.S4.x + sums.S4.y;
+        const float S5 = sums.S5.x + sums.S5.y, S6 = sums.S6.x + sums.S6.y;
         const float b1 = 0.5f * S2;
         const float c1 = S2 + fmaf(T3, -0.5f, fmaf(T4, 0.25f, fmaf(T5, -0.125f, T6 * 0.0625f)));
         const float c = S2 + fmaf(T3, -0.5f, fmaf(T4, 1.0f / 3.0f, fmaf(T5, -0.25f, T6 * 0.2f)));

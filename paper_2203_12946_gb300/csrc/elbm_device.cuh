@@ -610,6 +610,31 @@ __device__ __forceinline__ float2 opaque(float2 v)
     return v;
 }
 
+// The power sums M_k = <f, x^k> of all populations and S_k of those with x < 0 (Omega-), per
+// lane.  x^3 to x^6 share the products g2 = f x^2, g4 = f x^4, min(x, 0) and x min(x, 0), so the
+// nine sums take 13 paired operations instead of the 16 of separate powers of min(x, 0).  The
+// terms of each S_k have one sign: its error is a few units of itself, however small Omega- is
+// next to Omega+ (S_k as (M_k - <f, x^(k-1) |x|>) / 2 loses that; us per step of developed flows so
+// and here, 203 x 150 x 131 FP32 153.8, 157.7, 176 x 144 x 160 FP16 153.9, 157.1).
+struct PowerSums {
+    float2 M2 = f2(0.0f), M3 = f2(0.0f), M4 = f2(0.0f), M5 = f2(0.0f), M6 = f2(0.0f);
+    float2 S3 = f2(0.0f), S4 = f2(0.0f), S5 = f2(0.0f), S6 = f2(0.0f);
+    __device__ __forceinline__ void add(float2 f, float2 x)
+    {
+        const float2 x2 = pmul(x, x), g2 = pmul(f, x2), g4 = pmul(g2, x2);
+        const float2 xm = f2(fminf(x.x, 0.0f), fminf(x.y, 0.0f)), xxm = pmul(x, xm);
+        M2 = padd(M2, g2);
+        M3 = pfma(g2, x, M3);
+        M4 = padd(M4, g4);
+        M5 = pfma(g4, x, M5);
+        M6 = pfma(g4, x2, M6);
+        S3 = pfma(g2, xm, S3);
+        S4 = pfma(g2, xxm, S4);
+        S5 = pfma(g4, xm, S5);
+        S6 = pfma(g4, xxm, S6);
+    }
+};
+
 template <int D, bool kRelax = true, bool kDev = false, class PA>
 __device__ __forceinline__ float node_collide_pairs(PA &pa, float2 (&xp)[Pairs<D>::NP], const CollideParams &p,
                                                     int *branch)
@@ -790,36 +815,17 @@ __device__ __forceinline__ float node_collide_pairs(PA &pa, float2 (&xp)[Pairs<D
             sc = m2 + fmaf(m3, -0.5f, m4 * (1.0f / 3.0f));
             s3 = S3.x + S3.y, s4 = S4.x + S4.y;
         } else if (series) {
-            // Omega- through |x|: with A_k = <f, x^(k-1) |x|>, S_k = (M_k - A_k) / 2 for odd
-            // k, and A_k = <f, x^(k-2) x |x|> gives the same for even k.  M_k and A_k share
-            // the products g2 = f x^2, g4 = f x^4 and x |x|, so the nine sums take 13 paired
-            // operations instead of the 16 of separate powers of min(x, 0); the halves add
-            // numbers of the size of S_k itself, so nothing is lost to cancellation.
-            float2 M2 = f2(0.0f), M3 = f2(0.0f), M4 = f2(0.0f), M5 = f2(0.0f), M6 = f2(0.0f);
-            float2 A3 = f2(0.0f), A4 = f2(0.0f), A5 = f2(0.0f), A6 = f2(0.0f);
+            PowerSums sums;
 #pragma unroll
-            for (int k = 0; k < NP; ++k) {
-                const float2 xi = xp[k], x2 = pmul(xi, xi);
-                const float2 g2 = pmul(fagain(k), x2); // f x^2
-                const float2 g4 = pmul(g2, x2);        // f x^4
-                const float2 ax = f2(fabsf(xi.x), fabsf(xi.y)), xax = pmul(xi, ax);
-                M2 = padd(M2, g2);
-                M3 = pfma(g2, xi, M3);
-                M4 = padd(M4, g4);
-                M5 = pfma(g4, xi, M5);
-                M6 = pfma(g4, x2, M6);
-                A3 = pfma(g2, ax, A3);
-                A4 = pfma(g2, xax, A4);
-                A5 = pfma(g4, ax, A5);
-                A6 = pfma(g4, xax, A6);
-            }
-            const float m2 = M2.x + M2.y;
-            m3 = M3.x + M3.y, m4 = M4.x + M4.y, m5 = M5.x + M5.y, m6 = M6.x + M6.y;
+            for (int k = 0; k < NP; ++k) sums.add(fagain(k), xp[k]);
+            const float m2 = sums.M2.x + sums.M2.y;
+            m3 = sums.M3.x + sums.M3.y, m4 = sums.M4.x + sums.M4.y;
+            m5 = sums.M5.x + sums.M5.y, m6 = sums.M6.x + sums.M6.y;
+            s3 = sums.S3.x + sums.S3.y, s4 = sums.S4.x + sums.S4.y;
+            s5 = sums.S5.x + sums.S5.y, s6 = sums.S6.x + sums.S6.y;
             sb1 = 0.5f * m2;
             sc1 = m2 + fmaf(m3, -0.5f, fmaf(m4, 0.25f, fmaf(m5, -0.125f, m6 * 0.0625f))); // <f, 2x^2/(2+x)>
             sc = m2 + fmaf(m3, -0.5f, fmaf(m4, 1.0f / 3.0f, fmaf(m5, -0.25f, m6 * 0.2f)));
-            s3 = 0.5f * (m3 - (A3.x + A3.y)), s4 = 0.5f * (m4 - (A4.x + A4.y));
-            s5 = 0.5f * (m5 - (A5.x + A5.y)), s6 = 0.5f * (m6 - (A6.x + A6.y));
         } else {
             float2 b1 = f2(0.0f), c1 = f2(0.0f), c = f2(0.0f);
             float2 S3 = f2(0.0f), S4 = f2(0.0f), S5 = f2(0.0f), S6 = f2(0.0f);
@@ -1105,30 +1111,16 @@ __device__ __forceinline__ float2 node_collide_x2(float2 (&f)[9], float2 (&x)[9]
             sc = padd(M2, pfma(m3, f2(-0.5f), pmul(m4, f2(1.0f / 3.0f))));
             s3 = S3, s4 = S4;
         } else if (series) {
-            // Omega- sums through |x| (node_collide_pairs)
-            float2 M2 = f2(0.0f), A3 = f2(0.0f), A4 = f2(0.0f), A5 = f2(0.0f), A6 = f2(0.0f);
+            PowerSums sums; // both lanes' nodes
 #pragma unroll
-            for (int i = 0; i < Q; ++i) {
-                const float2 xi = x[i], x2 = pmul(xi, xi);
-                const float2 g2 = pmul(fagain(i), x2);
-                const float2 g4 = pmul(g2, x2);
-                const float2 ax = f2(fabsf(xi.x), fabsf(xi.y)), xax = pmul(xi, ax);
-                M2 = padd(M2, g2);
-                m3 = pfma(g2, xi, m3);
-                m4 = padd(m4, g4);
-                m5 = pfma(g4, xi, m5);
-                m6 = pfma(g4, x2, m6);
-                A3 = pfma(g2, ax, A3);
-                A4 = pfma(g2, xax, A4);
-                A5 = pfma(g4, ax, A5);
-                A6 = pfma(g4, xax, A6);
-            }
+            for (int i = 0; i < Q; ++i) sums.add(fagain(i), x[i]);
+            const float2 M2 = sums.M2;
+            m3 = sums.M3, m4 = sums.M4, m5 = sums.M5, m6 = sums.M6;
+            s3 = sums.S3, s4 = sums.S4, s5 = sums.S5, s6 = sums.S6;
             sb1 = pmul(f2(0.5f), M2);
             // <f, 2x^2/(2+x)> and c, Horner in the power sums
             sc1 = padd(M2, pfma(m3, f2(-0.5f), pfma(m4, f2(0.25f), pfma(m5, f2(-0.125f), pmul(m6, f2(0.0625f))))));
             sc = padd(M2, pfma(m3, f2(-0.5f), pfma(m4, f2(1.0f / 3.0f), pfma(m5, f2(-0.25f), pmul(m6, f2(0.2f))))));
-            s3 = pmul(f2(0.5f), psub(m3, A3)), s4 = pmul(f2(0.5f), psub(m4, A4));
-            s5 = pmul(f2(0.5f), psub(m5, A5)), s6 = pmul(f2(0.5f), psub(m6, A6));
         } else {
             float2 b1 = f2(0.0f), c1 = f2(0.0f), c = f2(0.0f), S3 = f2(0.0f), S4 = f2(0.0f), S5 = f2(0.0f),
                    S6 = f2(0.0f);

@@ -81,6 +81,24 @@ def test_fp64_square_root_is_ieee(probe):
     assert same(out, ieee)
 
 
+@pytest.mark.parametrize("share", [0.5, 0.1, 0.01])
+@pytest.mark.parametrize("q", [9, 27])
+def test_sums_over_omega_minus_keep_their_digits(probe, q, share):
+    """S_3..S_6, the sums of f x^k over x < 0, whose terms have one sign: within four roundings of
+    a term and one of each addition of their exact value, however small the negative departures are
+    next to the positive ones."""
+    rng = np.random.default_rng(q)
+    n = 4096
+    f = (rng.uniform(0.2, 1.0, (q, n)) / q).astype(np.float32)
+    x = rng.uniform(1e-3, 0.04, (q, n)) * np.where(rng.random((q, n)) < 0.5, 1.0, -share)
+    x = x.astype(np.float32)
+    (got,) = probe("probe_power_sums", [f, x], [((4, n), np.float32)], n, q)
+    fd, xm = f.astype(np.float64), np.minimum(x.astype(np.float64), 0.0)
+    for j in range(4):
+        want = (fd * xm ** (3 + j)).sum(0)
+        assert np.all(np.abs(got[j] - want) <= (4 + (q + 1) // 2 + 1) * 2.0 ** -24 * np.abs(want)), 3 + j
+
+
 @pytest.mark.parametrize("storage", ["f16dev", "bf16dev"])
 @pytest.mark.parametrize("D,dims", [(2, (1, 1, 1)), (2, (523, 301, 1)), (3, (41, 33, 29))])
 def test_16_bit_start_is_rounded_once(D, dims, storage):
