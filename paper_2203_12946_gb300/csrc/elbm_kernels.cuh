@@ -1388,7 +1388,8 @@ __global__ void __launch_bounds__(adjoint_block<ST>(), sizeof(typename ST::T) ==
 // Kinetic energy L = 1/2 sum rho |u|^2 of a stored field (FP64 sum into acc[0])
 // and, optionally, its gradient dL/df_i = c_i . u - |u|^2 / 2.  The FP32-arithmetic storages
 // take rho and rho u from exact_sums and form the gradient in double-float, rounded once to
-// FP32: 4.8 M D3Q27 nodes with gradient 207 us, where FP64 sums and gradients kept the FP64
+// FP32, or in FP64 where that is not sure to round alike (a node in some 10^4): 4.8 M D3Q27 nodes
+// with gradient 284 us (214 without the test, which is wrong where an entry cancels), where FP64 sums and gradients kept the FP64
 // pipe busy for 2.38 ms; 137 k nodes 15 (84), 65 k D2Q9 nodes 11 (26).
 template <class ST>
 __global__ void __launch_bounds__(kAuxBlock, 4) k_kinetic_energy(const typename ST::S *f, Geometry g, float Rf, double Rsum,
@@ -1414,8 +1415,23 @@ __global__ void __launch_bounds__(kAuxBlock, 4) k_kinetic_energy(const typename 
                 e = fma(0.5 * r, uu, e);
                 if (grad) {
                     DF ud[3], base = df_mulf(df_from_double(uu), -0.5f);
+                    float size = -base.hi;
 #pragma unroll
-                    for (int a = 0; a < D; ++a) ud[a] = df_from_double(u[a]);
+                    for (int a = 0; a < D; ++a) {
+                        ud[a] = df_from_double(u[a]);
+                        size += fabsf(ud[a].hi);
+                    }
+                    // stores an entry; its rounding is sure where what the sum leaves of the FP32
+                    // number is further than its error, below 2^-42 of the largest sum, from half
+                    // a unit in the last place
+                    bool sure = true;
+                    const float slack = 0x1p-42f * size;
+                    auto put = [&](int i, DF v) {
+                        grad[(int64_t)i * g.N + n] = v.hi;
+                        const uint32_t expo = __float_as_uint(v.hi) & 0x7f800000u;
+                        const float half = __uint_as_float(max(expo, 24u << 23) - (24u << 23));
+                        sure = sure && fabsf(fabsf(v.lo) - half) >= slack;
+                    };
                     auto along = [](DF b, DF w, int c) { return c == 0 ? b : df_add(b, c > 0 ? w : df_neg(w)); };
 #pragma unroll
                     for (int x = 0; x < 3; ++x) {
@@ -1424,12 +1440,20 @@ __global__ void __launch_bounds__(kAuxBlock, 4) k_kinetic_energy(const typename 
                         for (int y = 0; y < 3; ++y) {
                             const DF by = along(bx, ud[1], y - 1);
                             if constexpr (D == 2) {
-                                grad[(int64_t)(3 * x + y) * g.N + n] = by.hi;
+                                put(3 * x + y, by);
                             } else {
 #pragma unroll
-                                for (int z = 0; z < 3; ++z)
-                                    grad[(int64_t)(9 * x + 3 * y + z) * g.N + n] = along(by, ud[2], z - 1).hi;
+                                for (int z = 0; z < 3; ++z) put(9 * x + 3 * y + z, along(by, ud[2], z - 1));
                             }
+                        }
+                    }
+                    if (!sure) { // in FP64 (c . u and |u|^2 / 2 may cancel to any degree)
+#pragma unroll
+                        for (int i = 0; i < Q; ++i) {
+                            double cu = 0.0;
+#pragma unroll
+                            for (int a = 0; a < D; ++a) cu += vel(D, i, a) * u[a];
+                            grad[(int64_t)i * g.N + n] = T(cu - 0.5 * uu);
                         }
                     }
                 }

@@ -119,3 +119,31 @@ def test_16_bit_start_is_rounded_once(D, dims, storage):
         got = (got.astype(np.uint32) << 16).view(np.float32).astype(np.float64)
         unit = 2.0 ** (np.floor(np.log2(np.maximum(np.abs(got), 2.0 ** -126))) - 7)
     assert np.all(np.abs(got - (want - dev_ref(D)[:, None])) <= 0.5 * unit + 2.0 ** -44 * want)
+
+
+@pytest.mark.parametrize("storage", ["f32", "f32dev"])
+@pytest.mark.parametrize("D,dims", [(2, (251, 200, 1)), (3, (41, 33, 29))])
+def test_kinetic_energy_gradient_where_it_cancels(D, dims, storage):
+    """dL/df_i = c_i . u - |u|^2 / 2 with u on the circle (sphere) where it vanishes for one c_i, to
+    the rounding of the state: half a unit in the last place of the FP32 entry, and the few FP64
+    roundings of u and of the sum (2^-50 of its terms)."""
+    rng = np.random.default_rng(23)
+    N = int(np.prod(dims))
+    ux, uz = rng.uniform(-0.1, 0.1, N), rng.uniform(-0.05, 0.05, N) * (D == 3)
+    u = np.stack([ux, 1.0 - np.sqrt(1.0 + 2.0 * ux - ux * ux - uz * uz), uz])[:D]
+    f = O.init_equilibrium(D, rng.uniform(0.9, 1.1, N), u)
+    c = dev_ref(D)[:, None] if storage == "f32dev" else np.zeros((1, 1))
+    raw = (f - c).astype(np.float32)
+    with E.Simulation(LAT[D], dims, 0.97, storage=storage) as sim:
+        sim.set_populations(raw)
+        got = sim.kinetic_energy(with_grad=True)[1].cpu().numpy()
+    F = c.astype(np.longdouble) + raw.astype(np.longdouble)
+    vel = [[(i // 3 ** (D - 1 - a)) % 3 - 1 for a in range(D)] for i in range(3 ** D)]
+    rho = F.sum(0)
+    v = [sum(ci[a] * F[i] for i, ci in enumerate(vel)) / rho for a in range(D)]
+    uu = sum(w * w for w in v)
+    size = (sum(np.abs(w) for w in v) + uu).astype(np.float64)
+    for i, ci in enumerate(vel):
+        want = sum(ci[a] * v[a] for a in range(D)) - uu / 2
+        tol = 0.5 * np.spacing(np.abs(got[i])).astype(np.float64) + 2.0 ** -50 * size
+        assert np.all(np.abs(got[i].astype(np.longdouble) - want) <= tol), ci
