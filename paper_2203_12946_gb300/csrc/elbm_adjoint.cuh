@@ -330,7 +330,7 @@ __device__ void node_vjp(const T (&F)[Lattice<D>::Q], const T (&gin0)[Lattice<D>
 }
 
 // ---------------------------------------------------------------------------
-// FP32 vector-Jacobian product of one node's collision where |x|max < 0.04.
+// FP32 vector-Jacobian product of one node's collision where |x|max < kSeriesX.
 //
 // There alpha depends on the populations through the power sums M_k = <f, x^k> and, over
 // Omega-, S_k alone (node_collide_pairs), so with the adjoints m_k and s_k of the sums
@@ -486,7 +486,11 @@ __device__ __forceinline__ bool node_vjp_series(const float (&F)[Lattice<D>::Q],
         xabs = fmaxf(xabs, fmaxf(fabsf(x[k].x), fabsf(x[k].y)));
     }
     const bool lbgk = p.mode == kModeLBGK;
-    if (!lbgk && !(xabs < 0.04f)) return false;
+    if (!lbgk && !(xabs < kSeriesX)) return false;
+    if (lbgk) { // alpha is constant: no departure enters, however small a population is next to f^eq
+#pragma unroll
+        for (int k = 0; k < NP; ++k) x[k] = f2(0.0f);
+    }
 
     if constexpr (kForce) {
         // g <- (I + dPhi/df*)^T g, Phi the body-force term, and d<g, C + Phi>/dF_b

@@ -610,6 +610,10 @@ __device__ __forceinline__ float2 opaque(float2 v)
     return v;
 }
 
+// |x|max below which the path length's coefficients, and their derivatives in the reverse step,
+// are power series to x^6, and to x^4 (node_collide_pairs).
+constexpr float kSeriesX = 0.04f, kShortX = 0.005f;
+
 // The power sums M_k = <f, x^k> of all populations and S_k of those with x < 0 (Omega-), per
 // lane.  x^3 to x^6 share the products g2 = f x^2, g4 = f x^4, min(x, 0) and x min(x, 0), so the
 // nine sums take 13 paired operations instead of the 16 of separate powers of min(x, 0).  The
@@ -790,7 +794,6 @@ __device__ __forceinline__ float node_collide_pairs(PA &pa, float2 (&xp)[Pairs<D
         // rounding, so which one a lane gets moves its path length by less than that).
         // The scalar tail (sums to path length) spells its fused multiply-adds out, so that every
         // kernel this is inlined into rounds alike.
-        constexpr float kSeriesX = 0.04f, kShortX = 0.005f;
         const int form = __reduce_max_sync(__activemask(), xabs < kShortX ? 0 : (xabs < kSeriesX ? 1 : 2));
         const bool series = form < 2;
         float sb1, sc1, sc, s3, s4, s5 = 0.0f, s6 = 0.0f, m3 = 0.0f, m4 = 0.0f, m5 = 0.0f, m6 = 0.0f;
@@ -1086,7 +1089,6 @@ __device__ __forceinline__ float2 node_collide_x2(float2 (&f)[9], float2 (&x)[9]
     if (need[0] || need[1]) {
         // Coefficient forms of node_collide_pairs: x^4 series below kShortX, x^6 series
         // below kSeriesX, per-population rational terms above; one form per warp.
-        constexpr float kSeriesX = 0.04f, kShortX = 0.005f;
         auto form_of = [&](int l) { return !need[l] ? 0 : (xabs[l] < kShortX ? 0 : (xabs[l] < kSeriesX ? 1 : 2)); };
         const int form = __reduce_max_sync(__activemask(), max(form_of(0), form_of(1)));
         const bool series = form < 2;
