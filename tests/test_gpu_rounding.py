@@ -1,6 +1,7 @@
 """How results are rounded: where a value is formed in more bits than it is stored in, or by a
 division or root of the library's own, it is the correctly rounded one."""
 import ctypes
+import math
 import os
 import subprocess
 
@@ -18,15 +19,21 @@ pytestmark = pytest.mark.gpu
 
 @pytest.fixture(scope="module")
 def probe(tmp_path_factory):
-    """Calls a function of device_probes.cu, built with the library's flags: arrays go in as
-    device copies, the outputs (shape, dtype) come back as arrays."""
+    """Calls a function of device_probes.cu, or with D of lattice_probes.cu, built with the
+    library's flags: arrays go in as device copies, the outputs (shape, dtype) come back as arrays."""
     torch = pytest.importorskip("torch")
-    lib = str(tmp_path_factory.mktemp("probes") / "probes.so")
-    src = os.path.join(os.path.dirname(os.path.abspath(__file__)), "device_probes.cu")
-    subprocess.run([B.nvcc(), *B.ARCH, *B.NVCC_FLAGS, "-shared", "-o", lib, src, "-cudart", "static"], check=True)
-    so = ctypes.CDLL(lib)
+    libs = {}
 
-    def call(name, ins, outs, *scalars):
+    def load(D):
+        if D not in libs:
+            lib = str(tmp_path_factory.mktemp("probes") / f"probes{D}.so")
+            src = os.path.join(os.path.dirname(os.path.abspath(__file__)), "lattice_probes.cu" if D else "device_probes.cu")
+            subprocess.run([B.nvcc(), *B.ARCH, *B.NVCC_FLAGS, f"-DELBM_DIM={D}", "-shared", "-o", lib, src, "-cudart", "static"], check=True)
+            libs[D] = ctypes.CDLL(lib)
+        return libs[D]
+
+    def call(name, ins, outs, *scalars, D=0):
+        so = load(D)
         a = [torch.from_numpy(np.ascontiguousarray(v)).cuda() for v in ins]
         o = [torch.from_numpy(np.zeros(shape, dtype)).cuda() for shape, dtype in outs]
         torch.cuda.synchronize()
@@ -79,6 +86,61 @@ def test_fp64_square_root_is_ieee(probe):
     with np.errstate(all="ignore"):
         assert same(ieee, np.sqrt(a))
     assert same(out, ieee)
+
+
+def test_fp64_reciprocal_of_the_density(probe):
+    """1/rho of the moments: r0 (1 + e + e^2) with |e| < 2^-22 is off by 2^-66 of it before its one
+    rounding, against 2^-53 or more between two numbers: within one unit in the last place of the
+    correctly rounded reciprocal, and that reciprocal but for one density in 2^12 at most; what the
+    FP32 range cannot take is IEEE."""
+    rng = np.random.default_rng(3)
+    n = 1 << 20
+    edges = np.concatenate([EDGES, -EDGES])
+    rho = np.concatenate([rng.uniform(0.5, 2.0, n), doubles(rng, n, -120, 120), edges])
+    (out,) = probe("probe_rcp64", [rho], [(rho.shape, np.float64)], rho.size, D=2)
+    with np.errstate(all="ignore"):
+        want = 1.0 / rho
+    fp32 = (np.abs(rho) > 1e-30) & (np.abs(rho) < 1e30)
+    assert np.all(np.abs(out[fp32] - want[fp32]) <= np.spacing(np.abs(want[fp32])))
+    assert np.count_nonzero(out[fp32] != want[fp32]) <= 2 * n >> 12
+    assert same(out[~fp32], want[~fp32])
+
+
+@pytest.mark.parametrize("dev", [False, True])
+@pytest.mark.parametrize("D", [2, 3])
+def test_node_sums_are_exact_at_the_edges_of_their_forms(probe, D, dev):
+    """rho and rho u of a node's FP32 values (deviations: with the reference) are the exact sums
+    rounded once, by the split into two parts (up to 15 binades between a node's values, the
+    largest in 2^-63 .. 2^65) and by the fixed-point form past it: values over 0 to 20 binades,
+    exactly 15 and 16, all at the top of a binade, zeros among them, largest values on both sides
+    of the range; not-finite values are refused."""
+    rng = np.random.default_rng(31)
+    Q, n = 3 ** D, 512
+    top = np.float32(2.0 - 2.0 ** -23)  # largest significand
+
+    def spread(b, at=-4):
+        v = np.ldexp(rng.uniform(1.0, 2.0, (Q, n)), at - rng.integers(0, b + 1, (Q, n)))
+        v[0], v[-1] = np.ldexp(rng.uniform(1.0, 2.0, n), at), np.ldexp(rng.uniform(1.0, 2.0, n), at - b)
+        return v * rng.choice([-1.0, 1.0], (Q, n))
+
+    blocks = [spread(b) for b in (0, 1, 8, 14, 15, 16, 17, 20)]
+    blocks += [np.full((Q, n), 0.25) * top, np.full((Q, n), -0.25) * top, 0.25 * top * rng.choice([-1.0, 1.0], (Q, n))]
+    blocks += [spread(15) * (rng.random((Q, n)) < p) for p in (0.9, 0.5, 0.1, 0.0)]
+    low, high = (-14, 8) if dev else (-64, 66)  # binades of the largest value; 2^-63 and 2^64 end the split
+    blocks += [spread(b, at) for at in (low, low + 1, low + 2, high - 2, high - 1, high) for b in (0, 15, 16)]
+    v = np.concatenate(blocks, axis=1).astype(np.float32)
+    R = float(np.float32(6.0 ** -D)) if dev else 0.0
+    bad = np.repeat(v[:, :1], 3, axis=1)
+    bad[[0, Q // 2, Q - 1], [0, 1, 2]] = np.inf, np.nan, -np.inf
+    (out,) = probe("probe_exact_sums", [np.concatenate([v, bad], axis=1)], [((1 + D, v.shape[1] + 3), np.float64)],
+                   v.shape[1] + 3, ctypes.c_float(R), D=D)
+    assert np.all(out[:, -3:] == -1.0)
+    vel = np.array([[(i // 3 ** (D - 1 - a)) % 3 - 1 for a in range(D)] for i in range(Q)])
+    for k in range(v.shape[1]):
+        col = v[:, k].astype(np.float64)
+        assert out[0, k] == math.fsum([*col, 6 ** D * R]), k
+        for a in range(D):
+            assert out[1 + a, k] == math.fsum(vel[:, a] * col), (k, a)
 
 
 @pytest.mark.parametrize("share", [0.5, 0.1, 0.01])
