@@ -96,14 +96,16 @@ extern "C" {
 #define ELBM_B_DERIVED 0
 #define ELBM_B_PRINTED 1
 
-/* Kernel of elbm_step.  DIRECT: one node per thread, neighbours loaded
- * through the L1 cache; any dims.  ROWS: persistent CTAs stage every source
- * row of an x-row in shared memory with bulk asynchronous copies (TMA engine,
- * mbarrier pipeline); needs FP32 or 16-bit storage, nx * element size a
- * multiple of 16 bytes and nx <= 1024 (D2Q9) or 512 (D3Q27).  AUTO (default)
- * takes DIRECT, the faster of the two on GB300.  Both kernels evaluate the same
- * per-node arithmetic; they agree to rounding (the compiler may fuse
- * multiply-adds differently in each). */
+/* Kernel of elbm_step.  DIRECT: one node per thread (two in D2Q9 with FP32
+ * arithmetic), neighbours loaded through the L1 cache; any dims.  ROWS:
+ * persistent CTAs stage every source row of an x-row in shared memory with
+ * bulk asynchronous copies (TMA engine, mbarrier pipeline); needs FP32 or
+ * 16-bit storage, nx * element size a multiple of 16 bytes and nx <= 1024
+ * (D2Q9) or 512 (D3Q27).  AUTO (default) takes DIRECT, the faster of the two on
+ * GB300, or for small D2Q9 domains with FP32 arithmetic up to four of its steps
+ * in one launch (the same bits).  Both kernels evaluate the same per-node
+ * arithmetic; they agree to rounding (the compiler may fuse multiply-adds
+ * differently in each). */
 #define ELBM_KERNEL_AUTO 0
 #define ELBM_KERNEL_DIRECT 1
 #define ELBM_KERNEL_ROWS 2

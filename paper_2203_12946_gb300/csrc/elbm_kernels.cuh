@@ -4,9 +4,12 @@
 //
 //   k_step     fused pull-stream + collide + store (Eq. advection, Eq.
 //              fstar_def, path length of Sec. III / Appendix C-D), one node per
-//              thread, ping-pong buffers
-//   k_init     f = f^eq(rho, u) (Sec. I equilibrium, FP64, rounded to storage)
-//   k_moments  rho and u of the stored state (FP64; exact fixed-point sums of FP32 values)
+//              thread (D2Q9 in FP32 arithmetic: two), ping-pong buffers
+//   k_step_tile  several steps of a small D2Q9 domain in shared memory
+//   k_init     f = f^eq(rho, u) (Sec. I equilibrium, in FP64 or, for the FP32-arithmetic
+//              storages, in double-float; rounded once to storage)
+//   k_moments  rho and u of the stored state (FP64; exact sums of FP32 values, split into
+//              two FP32 parts or in fixed point)
 //   k_alpha    path length of the next collision (no write-back)
 //   k_diag     domain reductions: mass, momentum, H (Eq. hdef), alpha statistics
 //              and per-node H[f*] - H[f] (Eq. deltaH3) in FP64; warp shuffles,
@@ -658,8 +661,9 @@ __device__ __forceinline__ double rcp64(double rho)
 // FP64, the FP32-arithmetic storages by exact_sums (a node holding a value that is not finite
 // is summed in FP64).  4.8 M D3Q27 nodes of FP32 populations: 114 us = 5.9 TB/s (202 with
 // 64-bit fixed point for every value), FP32 deviations 133, FP16 131 (199); 8 M D2Q9 nodes 145,
-// 162, 162 (207, 237, 236; bound by the FP64 pipe).  At 48 registers (5 blocks of 256) rather than
-// the 80 the compiler takes: 141 us, too few loads in flight.
+// 162, 162 (207, 237, 236; bound by the FP64 pipe).  Five blocks of 256 are asked for: at their 48
+// registers the D3Q27 sums spill 152 bytes, but without that bound too few loads are in flight
+// (same box: FP32 107 and 133 us, FP32 deviations 124 and 149, FP16 118 and 139; D2Q9 alike).
 template <class ST>
 __global__ void __launch_bounds__(kAuxBlock, 5) k_moments(const typename ST::S *f, Geometry g, float Rf, double Rsum,
                                                       double *rho_out, double *u_out, int64_t n0, int64_t count)
@@ -1701,6 +1705,11 @@ cudaError_t ELBM_CAT(launch_step, ELBM_SUFFIX)(int storage, const void *fin, voi
     }
     const uint64_t elems = uint64_t(Q) * uint64_t(g.N);
     const RowDiv rd = row_div(uint32_t(g.nx));
+    // Steps with a body force take element offsets at every size, and no L2 instantiation: the
+    // force's two equilibria make them 1.5 times as long and byte offsets give 1 to 4 % of that (us
+    // per step, elements and bytes: D3Q27 201 x 160 x 150 FP32 294, 287, FP32 deviations 295, 283, FP16
+    // 284, 277, 60 x 52 x 44 11.1, 10.9; D2Q9 4000 x 2000 FP32 161.6, 159.6), for five more kernels
+    // per lattice to build.
 #define ELBM_DIRECT_STEP(ADDR, GRID)                                                                   \
     if (forced) {                                                                                      \
         ELBM_STORAGE_SWITCH(storage, return launch(k_step<ST, (ADDR == kAddrBytes ? kAddrElems : ADDR), true>, \
