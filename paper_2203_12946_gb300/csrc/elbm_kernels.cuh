@@ -342,14 +342,18 @@ __device__ __forceinline__ DF df_fast_two_sum(float a, float b) // |a| >= |b|
 // An FP64 value as hi, the nearest FP32 number, and lo, the rest rounded to FP32, on the
 // integer pipe: a conversion or an FP64 addition occupies GB300's FP64 pipe for 16 cycles per
 // warp and SM, and four values converted through it (16 such instructions) bounded the whole
-// kernel.  Below 2^-74 lo, and below 2^-126 the value, is flushed to zero; values beyond
-// FP32's range, infinities and NaN give infinities and NaN.
+// kernel.  Below 2^-74, where lo is no normal FP32 number for some, the conversions; values
+// beyond FP32's range, infinities and NaN give infinities and NaN.
 __device__ __forceinline__ DF df_from_double(double x)
 {
     const uint64_t b = (uint64_t)__double_as_longlong(x);
     const uint32_t top = uint32_t(b >> 32), sign = top & 0x80000000u;
     const int e = int((top >> 20) & 0x7ffu) - 896; // FP32's biased exponent
-    if (e <= 0) return {__uint_as_float(sign), 0.0f};
+    if (e <= 52) {
+        if ((b << 1) == 0) return {__uint_as_float(sign), 0.0f};
+        const float h = __double2float_rn(x);
+        return {h, __double2float_rn(x - double(h))};
+    }
     if (e >= 255) { // NaN stays NaN, anything else is infinite
         const bool nan = (top & 0x7fffffffu) > 0x7ff00000u || ((top & 0x7fffffffu) == 0x7ff00000u && uint32_t(b) != 0);
         return {__uint_as_float(sign | (nan ? 0x7fc00000u : 0x7f800000u)), 0.0f};
@@ -359,8 +363,7 @@ __device__ __forceinline__ DF df_from_double(double x)
     const uint32_t m = (uint32_t(e) << 23) | (uint32_t(b >> 29) & 0x7fffffu), low = uint32_t(b) & 0x1fffffffu;
     const uint32_t up = low > 0x10000000u || (low == 0x10000000u && (m & 1u)) ? 1u : 0u;
     const float rest = float(int(low) - int(up << 29)); // in units of 2^(e - 127 - 52)
-    const float scale = e > 52 ? __uint_as_float(sign | (uint32_t(e - 52) << 23)) : 0.0f;
-    return {__uint_as_float(sign | (m + up)), rest * scale};
+    return {__uint_as_float(sign | (m + up)), rest * __uint_as_float(sign | (uint32_t(e - 52) << 23))};
 }
 __device__ __forceinline__ DF df_add(DF a, DF b)
 {

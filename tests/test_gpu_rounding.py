@@ -209,3 +209,17 @@ def test_kinetic_energy_gradient_where_it_cancels(D, dims, storage):
         want = sum(ci[a] * v[a] for a in range(D)) - uu / 2
         tol = 0.5 * np.spacing(np.abs(got[i])).astype(np.float64) + 2.0 ** -50 * size
         assert np.all(np.abs(got[i].astype(np.longdouble) - want) <= tol), ci
+
+
+@pytest.mark.parametrize("D,dims", [(2, (131, 40, 1)), (3, (21, 13, 9))])
+def test_fp32_start_of_thin_matter_is_rounded_once(D, dims):
+    """As test_fp32_start_is_rounded_once (test_gpu_dispatch), for densities of 1e-28 to 1e-20, whose
+    second FP32 part is small but counts."""
+    N = int(np.prod(dims))
+    rng = np.random.default_rng(37)
+    rho, u = 10.0 ** rng.uniform(-28, -20, N), 0.08 * rng.standard_normal((D, N))
+    want = O.init_equilibrium(D, rho, u)
+    with E.Simulation(LAT[D], dims, 0.97, storage="f32") as sim:
+        sim.init_equilibrium(rho, u)
+        got = sim.get_populations()
+    assert np.all(np.abs(got - want) <= 0.5 * np.spacing(got).astype(np.float64) + 2.0 ** -44 * want)
