@@ -71,12 +71,14 @@ __device__ __forceinline__ void node_coords(int64_t n, const Geometry &g, int &x
 // nodes per thread (D2Q9): blocks along x-rows, y = blockIdx.y; byte offsets there are 55.8
 // against 59.0 us per step (2048^2 FP32, developed flow) and 24.6 against 26.5 (1501 x 997,
 // FP32 and FP16 deviations), and leave the DRAM-bound shear layers as they were.
+// (Developed flows here and below, both sides, with the Omega- sums as half differences; the
+// direct sums of PowerSums add 1 to 2.5 % to each.)
 // Minimum resident blocks per SM requested from the register allocator for the direct step
 // kernel.  D3Q27 with FP32 storage: 7 blocks of 128 (72 registers).  A step from DRAM is bound
 // by the bytes in flight, and the extra resident warps outweigh the spills (256^3, Taylor-Green
 // start: 0.544 ms with 7 blocks, 0.551 with 6, 0.579 with 5, 0.566 with 8).  FP32 deviations: 6
 // (80 registers).  A step whose two buffers stay in the L2 is bound by instructions and latency
-// instead: 5 blocks there (kL2Blocks, up to 102 registers, no spills; us per step, 7 or 6 blocks
+// instead: 5 blocks there (kL2Blocks, up to 102 registers, 4 bytes of spills; us per step, 7 or 6 blocks
 // and 5, near-equilibrium and developed flow: FP32 32^3 3.20, 3.04 and 3.33, 3.07; 64^3 10.96,
 // 10.45 and 14.69, 14.01; 80^3 20.7, 20.5 and 27.5, 26.4; 96^3, beyond the L2, 34.1, 35.3 and
 // 44.8, 43.5; FP32 deviations 32^3 3.54, 3.24, 72^3 16.2, 15.2 and 21.6, 20.8).  The 16-bit
@@ -1399,7 +1401,7 @@ __global__ void __launch_bounds__(adjoint_block<ST>(), sizeof(typename ST::T) ==
 // take rho and rho u from exact_sums and form the gradient in double-float, rounded once to
 // FP32, or in FP64 where that is not sure to round alike (a node in some 10^4): 4.8 M D3Q27 nodes
 // with gradient 284 us (214 without the test, which is wrong where an entry cancels), where FP64 sums and gradients kept the FP64
-// pipe busy for 2.38 ms; 137 k nodes 15 (84), 65 k D2Q9 nodes 11 (26).
+// pipe busy for 2.38 ms; 137 k nodes 18 (84), 65 k D2Q9 nodes 8 (26).
 template <class ST>
 __global__ void __launch_bounds__(kAuxBlock, 4) k_kinetic_energy(const typename ST::S *f, Geometry g, float Rf, double Rsum,
                                                              double *__restrict__ acc, typename ST::T *grad)
